@@ -51,7 +51,7 @@ extern "C" {
    device pointers need the alignment of their element type. */
 
 #define TWA_F32          0   /* batched FP32 path: fused Stockham passes, realization pairs */
-#define TWA_F64_PLAIN    1   /* comparator: complex128, one realization per launch, no fusion */
+#define TWA_F64_PLAIN    1   /* complex128 fields, every value computed in FP64; all streams in each launch */
 
 /* Number of FP64 scalars written per instance per output by twa_moments / twa_run. */
 #define TWA_NSCALARS     8

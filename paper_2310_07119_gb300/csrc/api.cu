@@ -73,8 +73,11 @@ struct Inst {
     double* prt = nullptr;
     double* dker[3] = {nullptr, nullptr, nullptr};
     // FP64 path
-    double2* work64 = nullptr;
-    double2* spec64 = nullptr;
+    double2* work64 = nullptr;  // packed Poisson fields of w_pairs pairs (2D, 3D)
+    double2* spec64 = nullptr;  // spectra of spec_fields slots
+    int w_pairs = 0, spec_fields = 0;
+    double* run64 = nullptr;    // partial sums of run64_outs + 1 outputs of a whole 1D run
+    int run64_outs = 0;
     double* acc64 = nullptr;
     double* acc64m = nullptr;
     double* bad64 = nullptr;
@@ -865,55 +868,89 @@ Tables64 tables64(const Inst& I) {
     return t;
 }
 
-int poisson_f64(twa_handle* h, Inst& I, double2* f, cudaStream_t st) {
-    const Geom64 g = geom64(I);
-    const Tables64 t = tables64(I);
-    launch_f64_rho(f, I.work64, I.cells, st, &h->launches);
-    launch_f64_fft3(I.work64, g, t, false, st, &h->launches);
-    launch_f64_poisson_mul(I.work64, g, t, -h->p.C / (double)I.cells, st, &h->launches);
-    launch_f64_fft3(I.work64, g, t, true, st, &h->launches);
-    return 0;
-}
+double mulc64(const twa_handle* h, const Inst& I) { return -h->p.C / (double)I.cells; }
 
 int step_batch_f64(twa_handle* h, Inst& I, double2* psi, int n, cudaStream_t st) {
-    const Geom64 g = geom64(I);
-    const Tables64 t = tables64(I);
-    const double kh = h->p.dt / (2.0 * h->p.hbar_m), kf = h->p.dt / h->p.hbar_m;
-    for (int s = 0; s < I.n_slots; ++s) {
-        double2* f = psi + (size_t)s * I.cells;
-        RC(poisson_f64(h, I, f, st));
-        launch_f64_kick(f, I.work64, I.cells, kh, st, &h->launches);
-        for (int k = 0; k < n; ++k) {
-            launch_f64_fft3(f, g, t, false, st, &h->launches);
-            launch_f64_kinetic(f, g, t, st, &h->launches);
-            launch_f64_fft3(f, g, t, true, st, &h->launches);
-            RC(poisson_f64(h, I, f, st));
-            launch_f64_kick(f, I.work64, I.cells, (k == n - 1) ? kh : kf, st, &h->launches);
-        }
-    }
+    const double kick = h->p.dt / h->p.hbar_m;
+    if (I.mode == MODE_1D)
+        launch_f64_run1d(psi, I.n_slots, geom64(I), tables64(I), mulc64(h, I), kick, 1, n, nullptr, nullptr, nullptr, st,
+                         &h->launches);
+    else
+        launch_f64_steps(psi, I.work64, I.w_pairs, I.n_slots, geom64(I), tables64(I), mulc64(h, I), kick, n, st,
+                         &h->launches);
     return 0;
 }
 
 int moments_f64(twa_handle* h, Inst& I, double2* psi, const twa_moments_out* o, double* scalars, cudaStream_t st) {
-    const Geom64 g = geom64(I);
-    const Tables64 t = tables64(I);
     CU(cudaMemsetAsync(I.bad64, 0, sizeof(double), st));
     const bool modes = h->p.want_modes && I.spec64;
-    for (int s = 1; s < I.n_slots; ++s) {
-        double2* f = psi + (size_t)s * I.cells;
-        launch_f64_moments_accum(f, nullptr, I.cells, 0.0, s == 1, I.acc64, I.bad64, st, &h->launches);
-        if (modes) {
-            CU(cudaMemcpyAsync(I.spec64, f, I.cells * sizeof(double2), cudaMemcpyDeviceToDevice, st));
-            launch_f64_fft3(I.spec64, g, t, false, st, &h->launches);
-            launch_f64_modes_accum(I.spec64, I.cells, h->p.n_tot * I.dV / (double)I.cells, s == 1, I.acc64m, st,
-                                   &h->launches);
-        }
-    }
+    launch_f64_moments_accum(psi, I.cells, I.n_slots, I.acc64, I.bad64, st, &h->launches);
+    if (modes)
+        launch_f64_modes(psi, I.spec64, I.spec_fields, I.n_slots, geom64(I), tables64(I),
+                         h->p.n_tot * I.dV / (double)I.cells, I.acc64m, st, &h->launches);
     launch_f64_moments_finish(I.acc64, modes ? I.acc64m : nullptr, psi, I.cells, I.n_real,
                               1.0 / (2.0 * h->p.n_tot * I.dV), I.dV, (double)I.cells / (2.0 * h->p.n_tot),
                               o ? o->rho_mean : nullptr, o ? o->psi_mean : nullptr, o ? o->rho_cl : nullptr,
                               o ? o->nk_mean : nullptr, o ? o->nk_var : nullptr, I.part_r, I.part_m, I.bad64, scalars,
                               h->d_err, st, &h->launches);
+    return 0;
+}
+
+// Workspace of the FP64 path, all of it allocated with the handle (its calls can be captured): packed
+// Poisson fields and spectra for as many streams as fit 1 GB (at least one; grid rows bound them too),
+// and for 1D instances the partial sums of as many outputs as fit 16 MB (none when two do not).
+int alloc_f64(twa_handle* h, Inst& I) {
+    const double field = (double)I.cells * sizeof(double2);
+    const int most = (int)std::max(1.0, std::min(32768.0, (double)(1LL << 30) / field));
+    if (I.mode != MODE_1D) {
+        I.w_pairs = std::min(I.n_pairs, most);
+        RC(dalloc(h, &I.work64, (size_t)I.w_pairs * I.cells));
+    } else {
+        const double per_out = (double)I.n_real * (3.0 * I.cells + 1.0) + I.cells;
+        I.run64_outs = (int)std::min(1024.0, (double)(16 << 20) / (8.0 * per_out)) - 1;
+        if (I.run64_outs > 0) RC(dalloc(h, &I.run64, (size_t)(I.run64_outs + 1) * (size_t)per_out));
+    }
+    RC(dalloc(h, &I.acc64, (size_t)3 * I.cells));
+    RC(dalloc(h, &I.bad64, 1));
+    if (h->p.want_modes) {
+        I.spec_fields = std::min(I.n_real, most);
+        RC(dalloc(h, &I.spec64, (size_t)I.spec_fields * I.cells));
+        RC(dalloc(h, &I.acc64m, (size_t)2 * I.cells));
+    }
+    if (f64_prepare() != 0) return fail(h, TWA_ECUDA, "cudaFuncSetAttribute failed");
+    return 0;
+}
+
+// Whole 1D FP64 runs: every output's sums come out of the stepping launch (as run1d_all).
+bool run1d_f64_eligible(const twa_handle* h) {
+    for (const auto& I : h->in)
+        if (I.mode != MODE_1D || !I.run64) return false;
+    return true;
+}
+
+int run1d_f64(twa_handle* h, double2* psi, int n_out, int out_every, double* series, cudaStream_t st) {
+    const int ni = (int)h->in.size();
+    for (int i = 0; i < ni; ++i) {
+        Inst& I = h->in[i];
+        const long long N = I.cells, R = I.n_real;
+        double* part = I.run64;
+        double* part_cl = part + (size_t)(I.run64_outs + 1) * R * 3 * N;
+        double* part_bad = part_cl + (size_t)(I.run64_outs + 1) * N;
+        int done = 0;
+        do {
+            const int k = std::min(I.run64_outs, n_out - done);
+            launch_f64_run1d(psi + I.off, I.n_slots, geom64(I), tables64(I), mulc64(h, I), h->p.dt / h->p.hbar_m, k,
+                             out_every, part, part_cl, part_bad, st, &h->launches);
+            // the first launch reports its initial output; later ones start where the last one ended
+            const int skip = done == 0 ? 0 : 1;
+            launch_finish_run1d(part + skip * R * 3 * N, part_cl + skip * N, part_bad + skip * R, (int)R, (int)N,
+                                k + 1 - skip, 1.0 / (double)R, 1.0 / (2.0 * h->p.n_tot * I.dV), I.dV,
+                                (double)I.cells / (2.0 * h->p.n_tot), h->p.want_modes ? h->p.n_tot : 0.0, series,
+                                done + skip, i, ni, h->d_err, st);
+            ++h->launches;
+            done += k;
+        } while (done < n_out);
+    }
     return 0;
 }
 
@@ -932,7 +969,7 @@ int build_tables(twa_handle* h, Inst& I) {
             k2f[j] = (float)(k * k);
             double c, s;
             phase_of(hb * k * k * dt / 2.0, c, s);
-            phd[j] = make_double2(c, s);
+            phd[j] = make_double2(c / n, s / n);
             phf[j] = make_float2((float)(c / n), (float)(s / n));
             phl[j] = make_float2((float)(c / n - (double)phf[j].x), (float)(s / n - (double)phf[j].y));
             const double ang = -2.0 * M_PI * (double)j / (double)n;
@@ -1065,13 +1102,7 @@ int twa_create(twa_handle** out, const twa_grid* grids, const twa_params* p, int
             cudaMemset(I.vc, 0, (size_t)I.n_pairs * I.cells * sizeof(float2));
             if (p->want_modes && (rc = dalloc(h, &I.spec, (size_t)I.n_slots * I.cells))) return bail(rc);
         } else {
-            if ((rc = dalloc(h, &I.work64, (size_t)I.cells))) return bail(rc);
-            if ((rc = dalloc(h, &I.acc64, (size_t)3 * I.cells))) return bail(rc);
-            if ((rc = dalloc(h, &I.bad64, 1))) return bail(rc);
-            if (p->want_modes) {
-                if ((rc = dalloc(h, &I.spec64, (size_t)I.cells))) return bail(rc);
-                if ((rc = dalloc(h, &I.acc64m, (size_t)2 * I.cells))) return bail(rc);
-            }
+            if ((rc = alloc_f64(h, I))) return bail(rc);
         }
     }
     if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1367,6 +1398,11 @@ int twa_advance(twa_handle* h, void* psi_work, int n_steps, int out_every, doubl
     h->launches = 0;
     const int n_out = n_steps / out_every;
     CU(cudaMemsetAsync(h->d_counter, 0, sizeof(int), user));
+    if (h->p.precision == TWA_F64_PLAIN && run1d_f64_eligible(h)) {
+        RC(run1d_f64(h, static_cast<double2*>(psi_work), n_out, out_every, series, user));
+        CU(cudaGetLastError());
+        return TWA_OK;
+    }
     if (h->p.precision == TWA_F64_PLAIN) {
         for (int o = 0; o <= n_out; ++o) {
             if (o > 0) {

@@ -41,7 +41,7 @@ int launch_phase_moments(const float2* psi, long long cells, int n_slots, double
 int launch_phase_moments_f64(const double2* psi, long long cells, int n_slots, double weyl, double dV,
                              double* var_a, double* phi2, double* part, double* out, cudaStream_t st);
 
-// Plain FP64 comparator path (one realization per launch, no fusion).
+// FP64 path (plain_f64.cu).
 struct Geom64 {
     int dim;
     int n[3];
@@ -49,19 +49,22 @@ struct Geom64 {
 };
 struct Tables64 {
     const double2* tw[3];     // exp(-2 pi i m / n_a) per axis
-    const double2* ph[3];     // exp(-i hbar k_a^2 dt / 2) per axis (FFT order)
+    const double2* ph[3];     // exp(-i hbar k_a^2 dt / 2) / n_a per axis (FFT order)
     const double* k2[3];      // k_a^2 per axis
 };
-int launch_f64_fft3(double2* f, const Geom64& g, const Tables64& t, bool inverse, cudaStream_t st, long long* nl);
-int launch_f64_kinetic(double2* f, const Geom64& g, const Tables64& t, cudaStream_t st, long long* nl);
-int launch_f64_rho(const double2* psi, double2* work, long long cells, cudaStream_t st, long long* nl);
-int launch_f64_poisson_mul(double2* work, const Geom64& g, const Tables64& t, double mulc, cudaStream_t st,
-                           long long* nl);
-int launch_f64_kick(double2* psi, const double2* work, long long cells, double kick, cudaStream_t st, long long* nl);
-int launch_f64_moments_accum(const double2* psi, const double2* work, long long cells, double kick, int first,
-                             double* acc /*3*cells*/, double* bad, cudaStream_t st, long long* nl);
-int launch_f64_modes_accum(const double2* spec, long long cells, double anorm2, int first, double* acc2 /*2*cells*/,
-                           cudaStream_t st, long long* nl);
+int f64_prepare();            // kernel attributes of the current device; 0 or -3
+// n_steps KDK steps of a synchronized 2D or 3D batch, w_pairs pairs of streams at a time (W: w_pairs fields)
+int launch_f64_steps(double2* psi, double2* W, int w_pairs, int n_slots, const Geom64& g, const Tables64& t, double mulc,
+                     double kick, int n_steps, cudaStream_t st, long long* nl);
+// n_out intervals of out_every steps of a synchronized 1D batch; part (or null): [(n_out + 1) n_real][3][N],
+// part_cl [n_out + 1][N], part_bad [(n_out + 1) n_real], as launch_finish_run1d reads them
+int launch_f64_run1d(double2* psi, int n_slots, const Geom64& g, const Tables64& t, double mulc, double kick, int n_out,
+                     int out_every, double* part, double* part_cl, double* part_bad, cudaStream_t st, long long* nl);
+int launch_f64_moments_accum(const double2* psi, long long cells, int n_slots, double* acc /*3*cells*/, double* bad,
+                             cudaStream_t st, long long* nl);
+// sums of |a_k|^2 and |a_k|^4 over slots 1.., spec_fields transforms at a time
+int launch_f64_modes(const double2* psi, double2* spec, int spec_fields, int n_slots, const Geom64& g, const Tables64& t,
+                     double anorm2, double* acc2 /*2*cells*/, cudaStream_t st, long long* nl);
 int launch_f64_moments_finish(const double* acc, const double* acc2, const double2* psi0, long long cells, int n_real,
                               double weyl, double dV, double q_offset, double* rho_mean, double* psi_mean,
                               double* rho_cl, double* nk_mean, double* nk_var, double* part_r, double* part_m,

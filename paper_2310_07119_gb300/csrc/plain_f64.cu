@@ -1,8 +1,20 @@
-// plain_f64.cu - plain FP64 single-realization comparator path (complex128, no fusion).
+// plain_f64.cu - the FP64 path (complex128): the batched split step of Sec. III.B.2, Eq. mft_normed,
+// with every value held and computed in 64 bits.
 //
-// The same split step as the batched path (Sec. III.B.2, Eq. mft_normed) written the plain way:
-// every FFT axis, the kinetic phase, the density, the Poisson multiplier and the kick are separate
-// kernels, one realization per launch.  The FFT is a radix-2 Stockham transform of one line per CTA.
+// GB300 runs FP64 at 1/64 of its FP32 rate, so every kernel here is bound by FP64 issue, not by memory:
+// what counts is the number of FP64 instructions per value and that all SMs have work.
+//   * Line transforms are Stockham radix-4 (a radix-2 stage first when log2 N is odd) of butterflies
+//     a +- w b in six fused multiply-adds (a + w b, then 2 a - (a + w b)): 3 instructions per value and
+//     radix-2 level instead of 4.  Four values per thread, stages exchanged through shared memory.
+//   * Two streams share one complex Poisson transform (their densities are its real and imaginary
+//     part; the Poisson operator is real), and the kick, the kinetic phase, the density and 1/k^2 are
+//     part of the transform passes.
+//   * All streams of a batch run in each launch.  One launch per stream and operation left most SMs
+//     idle: 100 steps of 32 streams of 256 cells took 25,000 launches and 186 ms.
+//   * A 1D field stays on one SM for a whole run (k64_run1d), a stream per CTA.
+// Measured before and after (one GB300): 100 steps of 32 streams of 256 cells, moments every 10,
+// 182.6 -> 1.55 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.19 ms, where FP64 issue
+// alone (about 245 instructions per value and step at 2 per cycle and SM) takes 3.9 ms.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
@@ -14,119 +26,356 @@ __device__ __forceinline__ double2 zmul(double2 a, double2 b) {
     return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
 
-// One line of length N (stride S) per CTA; lines are (q, o) with base q + o OS, q < Qn.
-__global__ void k64_fft_line(double2* f, int N, long long S, int Qn, long long OS, const double2* __restrict__ tw,
-                             int inv) {
-    extern __shared__ double2 sm64[];
-    double2* a = sm64;
-    double2* b = sm64 + N;
-    const long long L = blockIdx.x;
-    const long long base = (L % Qn) + (L / Qn) * OS;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) a[i] = f[base + i * S];
-    __syncthreads();
-    for (int ns = 1; ns < N; ns *= 2) {
-        for (int j = threadIdx.x; j < N / 2; j += blockDim.x) {
-            const int k = j & (ns - 1);
-            double2 w = tw[k * (N / (2 * ns))];
-            if (inv) w.y = -w.y;
-            const double2 v0 = a[j];
-            const double2 v1 = zmul(a[j + N / 2], w);
-            const int d = (j / ns) * ns * 2 + k;
-            b[d] = make_double2(v0.x + v1.x, v0.y + v1.y);
-            b[d + ns] = make_double2(v0.x - v1.x, v0.y - v1.y);
-        }
+// (a, b) <- (a + w b, a - w b)
+__device__ __forceinline__ void bfly(double2& a, double2& b, double2 w) {
+    const double2 p = make_double2(fma(w.x, b.x, fma(-w.y, b.y, a.x)), fma(w.x, b.y, fma(w.y, b.x, a.y)));
+    b = make_double2(fma(2.0, a.x, -p.x), fma(2.0, a.y, -p.y));
+    a = p;
+}
+__device__ __forceinline__ void bfly1(double2& a, double2& b) {
+    const double2 d = make_double2(a.x - b.x, a.y - b.y);
+    a = make_double2(a.x + b.x, a.y + b.y);
+    b = d;
+}
+
+// Shared-memory slot of element i: one 16-byte slot of padding per 8 (the first stages store with
+// strides of two and four elements).
+__device__ __forceinline__ int pad64(int i) { return i + (i >> 3); }
+__host__ __device__ constexpr int line64(int n) { return n + n / 8 + 1; }
+
+// Transform of one line of N = 2^lg values by N / V threads: thread j holds elements j + r N / V, r < V,
+// before and after.  a and b: two exchange lines of line64(N), used in turn by every exchange of a kernel
+// (a line is written again only behind the barrier of the exchange in between, so each exchange has
+// one barrier); every thread of the CTA takes part.
+template <int V>
+__device__ __forceinline__ void fft64(double2 (&v)[V], int j, int N, int lg, bool inv, double2*& a, double2*& b,
+                                      const double2* __restrict__ tw) {
+    auto root = [&](int e) {
+        double2 w = __ldg(&tw[e]);
+        if (inv) w.y = -w.y;
+        return w;
+    };
+    auto exchange = [&](const int (&d)[V]) {
+#pragma unroll
+        for (int r = 0; r < V; ++r) a[pad64(d[r])] = v[r];
         __syncthreads();
+#pragma unroll
+        for (int r = 0; r < V; ++r) v[r] = a[pad64(j + r * (N / V))];
         double2* t = a;
         a = b;
         b = t;
+    };
+    int ns = 1;
+    if constexpr (V == 2) {
+#pragma unroll 1
+        for (; ns < N; ns *= 2) {
+            const int k = j & (ns - 1);
+            if (ns == 1) bfly1(v[0], v[1]);
+            else bfly(v[0], v[1], root(k * (N / (2 * ns))));
+            if (2 * ns < N) {
+                const int d = (j - k) * 2 + k;
+                exchange({d, d + ns});
+            }
+        }
+    } else {
+        const int q = N / 4;
+        if (lg & 1) {  // radix 2: the butterflies j and j + N / 4
+            bfly1(v[0], v[2]);
+            bfly1(v[1], v[3]);
+            exchange({2 * j, 2 * (j + q), 2 * j + 1, 2 * (j + q) + 1});
+            ns = 2;
+        }
+#pragma unroll 1
+        for (; ns < N; ns *= 4) {
+            const int k = j & (ns - 1), s = q / ns;
+            if (ns == 1) {
+                bfly1(v[0], v[2]);
+                bfly1(v[1], v[3]);
+                const double2 n = inv ? make_double2(-v[3].y, v[3].x) : make_double2(v[3].y, -v[3].x);
+                v[3] = n;
+                bfly1(v[0], v[1]);
+                bfly1(v[2], v[3]);
+            } else {
+                const double2 w1 = root(k * s), w2 = root(2 * k * s);
+                bfly(v[0], v[2], w2);
+                bfly(v[1], v[3], w2);
+                bfly(v[0], v[1], w1);
+                bfly(v[2], v[3], inv ? make_double2(-w1.y, w1.x) : make_double2(w1.y, -w1.x));
+            }
+            // v = outputs 0, 2, 1, 3 of the butterfly
+            const double2 t = v[1];
+            v[1] = v[2];
+            v[2] = t;
+            if (4 * ns < N) {
+                const int d = (j - k) * 4 + k;
+                exchange({d, d + ns, d + 2 * ns, d + 3 * ns});
+            }
+        }
     }
-    for (int i = threadIdx.x; i < N; i += blockDim.x) f[base + i * S] = a[i];
 }
 
-__device__ __forceinline__ void coords(long long e, const int* n, int& x, int& y, int& z) {
-    x = (int)(e % n[0]);
-    const long long r = e / n[0];
-    y = (int)(r % n[1]);
-    z = (int)(r / n[1]);
+// z exp(-i theta).  Up to 1/4 sin and cos are their Taylor sums (next terms below 1e-17 relative);
+// beyond, theta is reduced mod 2 pi in FP64.  sincos alone took three times the instructions.
+__device__ __forceinline__ double2 kick64(double2 z, double th) {
+    double s, c;
+    if (fabs(th) <= 0.25) {
+        const double t = th * th;
+        s = fma(t, fma(t, fma(t, fma(t, fma(t, -1.0 / 39916800.0, 1.0 / 362880.0), -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0) * th;
+        c = fma(t, fma(t, fma(t, fma(t, fma(t, fma(t, 1.0 / 479001600.0, -1.0 / 3628800.0), 1.0 / 40320.0), -1.0 / 720.0),
+                                     1.0 / 24.0), -0.5), 1.0);
+    } else {
+        const double two_pi = 6.283185307179586476925286766559;
+        sincos(th - two_pi * rint(th / two_pi), &s, &c);
+    }
+    return make_double2(fma(z.x, c, z.y * s), fma(z.y, c, -z.x * s));
 }
 
-struct G64 {
-    int n[3];
-    long long cells;
+// One axis of a pass: a CTA owns L lines of N = 2^lg values, N / 4 threads a line (power-of-two grids).
+struct Axis64 {
+    int N, lg, L;
+    int S;                       // stride of the axis
+    long long lines, cells;      // lines and cells of one field
+    const double2* tw;           // exp(-2 pi i m / N)
+    const double2* ph;           // exp(-i hbar k^2 dt / 2) / N
 };
 
-// f <- f exp(-i hbar k^2 dt / 2) / cells (product of the per-axis factors)
-__global__ void k64_kinetic(double2* f, G64 g, const double2* px, const double2* py, const double2* pz) {
-    const double sc = 1.0 / (double)g.cells;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < g.cells; e += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        coords(e, g.n, x, y, z);
-        const double2 ph = zmul(zmul(px[x], py[y]), pz[z]);
-        const double2 v = zmul(f[e], ph);
-        f[e] = make_double2(v.x * sc, v.y * sc);
+struct Line64 {
+    int j;
+    long long at;   // first element of the line in its field
+    int step;       // element distance of this thread's four values
+    bool act;
+    double2 *a, *b;
+};
+__device__ __forceinline__ Line64 line_of(const Axis64& x) {
+    extern __shared__ double2 sm64[];
+    Line64 l;
+    const int q = x.N / 4;
+    // consecutive threads walk along a contiguous line, across the lines of a strided axis
+    const int k = x.S == 1 ? threadIdx.x / q : threadIdx.x % x.L;
+    l.j = x.S == 1 ? threadIdx.x % q : threadIdx.x / x.L;
+    long long id = (long long)blockIdx.x * x.L + k;
+    l.act = id < x.lines;
+    if (!l.act) id = x.lines - 1;   // partial tiles of small grids run on a clamped line and store nothing
+    l.at = x.S == 1 ? id * x.N : (id % x.S) + (id / x.S) * x.S * x.N;
+    l.at += (long long)l.j * x.S;
+    l.step = q * x.S;
+    l.a = sm64 + (size_t)k * line64(x.N);
+    l.b = l.a + (size_t)x.L * line64(x.N);
+    return l;
+}
+__device__ __forceinline__ void load4(double2 (&v)[4], const double2* f, const Line64& l) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[r] = f[l.at + (long long)r * l.step];
+}
+__device__ __forceinline__ void store4(const double2 (&v)[4], double2* f, const Line64& l) {
+    if (!l.act) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) f[l.at + (long long)r * l.step] = v[r];
+}
+__device__ __forceinline__ void fft4(double2 (&v)[4], Line64& l, const Axis64& x, bool inv) {
+    fft64<4>(v, l.j, x.N, x.lg, inv, l.a, l.b, x.tw);
+}
+__device__ __forceinline__ void drift4(double2 (&v)[4], Line64& l, const Axis64& x) {
+    fft4(v, l, x, false);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[r] = zmul(v[r], __ldg(&x.ph[l.j + r * (x.N / 4)]));
+    fft4(v, l, x, true);
+}
+
+// Pair of slots (2p, 2p + 1), p = blockIdx.y: kick with the pair's potentials (re, im of W; spectral
+// along the axis if vinv), then, if drift, the axis' kinetic factor.
+__global__ void __launch_bounds__(512) k64_kick_drift(Axis64 x, double2* psi, const double2* __restrict__ W, int n_slots,
+                                                       double kick, int vinv, int drift) {
+    Line64 l = line_of(x);
+    double2 w[4], v[4];
+    load4(w, W + (long long)blockIdx.y * x.cells, l);
+    if (vinv) fft4(w, l, x, true);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const int slot = 2 * blockIdx.y + h;
+        if (slot >= n_slots) break;
+        double2* f = psi + (long long)slot * x.cells;
+        load4(v, f, l);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = kick64(v[r], kick * (h ? w[r].y : w[r].x));
+        if (drift) drift4(v, l, x);
+        store4(v, f, l);
     }
 }
 
-__global__ void k64_rho(const double2* psi, double2* work, long long cells) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cells; e += (long long)gridDim.x * blockDim.x) {
-        const double2 z = psi[e];
-        work[e] = make_double2(z.x * z.x + z.y * z.y, 0.0);
-    }
+__global__ void __launch_bounds__(512) k64_drift(Axis64 x, double2* psi) {
+    Line64 l = line_of(x);
+    double2 v[4];
+    double2* f = psi + (long long)blockIdx.y * x.cells;
+    load4(v, f, l);
+    drift4(v, l, x);
+    store4(v, f, l);
 }
 
-// V_k = -C rho_k / (k^2 cells), V_0 = 0
-__global__ void k64_poisson_mul(double2* w, G64 g, const double* kx, const double* ky, const double* kz, double mulc) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < g.cells; e += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        coords(e, g.n, x, y, z);
-        const double k2 = kx[x] + ky[y] + kz[z];
-        const double m = (k2 > 0.0) ? mulc / k2 : 0.0;
-        w[e] = make_double2(w[e].x * m, w[e].y * m);
-    }
-}
-
-// psi <- psi exp(-i kick V), V = Re(work); the phase is reduced mod 2 pi in FP64.
-__global__ void k64_kick(double2* psi, const double2* work, long long cells, double kick) {
-    const double two_pi = 6.283185307179586476925286766559;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cells; e += (long long)gridDim.x * blockDim.x) {
-        double th = kick * work[e].x;
-        th = th - two_pi * rint(th / two_pi);
-        double s, c;
-        sincos(th, &s, &c);
-        const double2 z = psi[e];
-        psi[e] = make_double2(z.x * c + z.y * s, z.y * c - z.x * s);
-    }
-}
-
-// Running per-cell sums over realizations (first = 1 initializes): acc = (sum |psi|^2, sum re, sum im).
-__global__ void k64_moments_accum(const double2* psi, long long cells, int first, double* acc, double* bad) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cells; e += (long long)gridDim.x * blockDim.x) {
-        const double2 z = psi[e];
-        const double m = z.x * z.x + z.y * z.y;
-        if (first) {
-            acc[e] = m;
-            acc[cells + e] = z.x;
-            acc[2 * cells + e] = z.y;
-        } else {
-            acc[e] += m;
-            acc[cells + e] += z.x;
-            acc[2 * cells + e] += z.y;
+// Pair: the axis' kinetic factor (if drift), then the packed densities transformed into W.
+__global__ void __launch_bounds__(512) k64_drift_rho(Axis64 x, double2* psi, double2* __restrict__ W, int n_slots,
+                                                      int drift) {
+    Line64 l = line_of(x);
+    double2 v[4], w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) w[r] = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const int slot = 2 * blockIdx.y + h;
+        if (slot >= n_slots) break;
+        double2* f = psi + (long long)slot * x.cells;
+        load4(v, f, l);
+        if (drift) {
+            drift4(v, l, x);
+            store4(v, f, l);
         }
-        if (!isfinite(z.x) || !isfinite(z.y)) atomicAdd(bad, 1.0);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const double d = fma(v[r].x, v[r].x, v[r].y * v[r].y);
+            if (h) w[r].y = d;
+            else w[r].x = d;
+        }
+    }
+    fft4(w, l, x, false);
+    store4(w, W + (long long)blockIdx.y * x.cells, l);
+}
+
+// One field src -> dst (which may be the same): forward (mode 0), inverse (1), or forward, Poisson
+// multiplier mulc / k^2 (0 at k = 0), inverse (2).
+__global__ void __launch_bounds__(512) k64_field(Axis64 x, const double2* src, double2* dst, int mode, int lx, int lxy,
+                                                  const double* __restrict__ kx, const double* __restrict__ ky,
+                                                  const double* __restrict__ kz, double mulc) {
+    Line64 l = line_of(x);
+    double2 v[4];
+    load4(v, src + (long long)blockIdx.y * x.cells, l);
+    fft4(v, l, x, mode == 1);
+    if (mode == 2) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const long long e = l.at + (long long)r * l.step;
+            const double k2 = __ldg(&kx[e & ((1 << lx) - 1)]) + __ldg(&ky[(e >> lx) & ((1 << (lxy - lx)) - 1)]) +
+                              __ldg(&kz[e >> lxy]);
+            const double m = k2 > 0.0 ? mulc / k2 : 0.0;
+            v[r] = make_double2(v[r].x * m, v[r].y * m);
+        }
+        fft4(v, l, x, true);
+    }
+    store4(v, dst + (long long)blockIdx.y * x.cells, l);
+}
+
+// A whole 1D run of one stream (slot blockIdx.x) on one SM: KDK steps with adjacent half kicks merged,
+// and at the start and after every out_every steps the synchronized field's |psi|^2, Re psi and Im psi
+// per cell (the classical slot: |psi|^2) into partial sums that k_finish_run1d adds over the streams.
+// FP64 issue bounds it (about 9 us a step at 256 cells; N / 2 threads up to 256 cells so that the four
+// schedulers of the SM all have a warp), and an exchange costs a barrier of a few warps.
+template <int V>
+__global__ void __launch_bounds__(512) k64_run1d(double2* psi, int N, int lg, const double2* __restrict__ tw,
+                                                 const double2* __restrict__ ph, const double* __restrict__ k2, double mulc,
+                                                 double kick, int n_out, int out_every, int n_real, double* part,
+                                                 double* part_cl, double* part_bad) {
+    extern __shared__ double2 sm64[];
+    double2 *a = sm64, *b = sm64 + line64(N);
+    const int j = threadIdx.x, q = N / V, slot = blockIdx.x;
+    double2* f = psi + (long long)slot * N;
+    double2 v[V], p[V];
+    double m[V], pot[V];
+#pragma unroll
+    for (int r = 0; r < V; ++r) {
+        v[r] = f[j + r * q];
+        p[r] = ph[j + r * q];
+        const double k = k2[j + r * q];
+        m[r] = k > 0.0 ? mulc / k : 0.0;
+    }
+    auto poisson = [&]() {
+        double2 w[V];
+#pragma unroll
+        for (int r = 0; r < V; ++r) w[r] = make_double2(fma(v[r].x, v[r].x, v[r].y * v[r].y), 0.0);
+        fft64<V>(w, j, N, lg, false, a, b, tw);
+#pragma unroll
+        for (int r = 0; r < V; ++r) w[r] = make_double2(w[r].x * m[r], w[r].y * m[r]);
+        fft64<V>(w, j, N, lg, true, a, b, tw);
+#pragma unroll
+        for (int r = 0; r < V; ++r) pot[r] = w[r].x;
+    };
+    auto output = [&](int o, double kk) {
+        if (!part) return;
+        int bad = 0;
+        double* pp = part + ((long long)o * n_real + slot - 1) * 3 * N;
+#pragma unroll
+        for (int r = 0; r < V; ++r) {
+            const int g = j + r * q;
+            const double d = fma(v[r].x, v[r].x, v[r].y * v[r].y);
+            if (slot == 0) {
+                part_cl[(long long)o * N + g] = d;
+                continue;
+            }
+            const double2 z = kk != 0.0 ? kick64(v[r], kk * pot[r]) : v[r];
+            pp[g] = d;
+            pp[N + g] = z.x;
+            pp[2 * N + g] = z.y;
+            bad += (!isfinite(z.x) || !isfinite(z.y)) ? 1 : 0;
+        }
+        int all = __syncthreads_count(bad > 0);
+        if constexpr (V > 1) all += __syncthreads_count(bad > 1);
+        if constexpr (V > 2) all += __syncthreads_count(bad > 2) + __syncthreads_count(bad > 3);
+        if (slot > 0 && j == 0) part_bad[(long long)o * n_real + slot - 1] = (double)all;
+    };
+    poisson();
+    output(0, 0.0);
+#pragma unroll 1
+    for (int o = 1; o <= n_out; ++o) {
+#pragma unroll 1
+        for (int s = 0; s < out_every; ++s) {
+            const double kk = (o == 1 && s == 0) ? 0.5 * kick : kick;
+#pragma unroll
+            for (int r = 0; r < V; ++r) v[r] = kick64(v[r], kk * pot[r]);
+            fft64<V>(v, j, N, lg, false, a, b, tw);
+#pragma unroll
+            for (int r = 0; r < V; ++r) v[r] = zmul(v[r], p[r]);
+            fft64<V>(v, j, N, lg, true, a, b, tw);
+            poisson();
+        }
+        output(o, 0.5 * kick);
+    }
+    if (n_out == 0) return;
+#pragma unroll
+    for (int r = 0; r < V; ++r) f[j + r * q] = kick64(v[r], 0.5 * kick * pot[r]);
+}
+
+// Per-cell sums over the streams, in slot order: acc = (sum |psi|^2, sum re, sum im).
+__global__ void k64_moments_accum(const double2* __restrict__ psi, long long cells, int n_slots, double* acc, double* bad) {
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cells; e += (long long)gridDim.x * blockDim.x) {
+        double m = 0.0, x = 0.0, y = 0.0;
+        int nb = 0;
+#pragma unroll 4
+        for (int s = 1; s < n_slots; ++s) {
+            const double2 z = psi[(long long)s * cells + e];
+            m += z.x * z.x + z.y * z.y;
+            x += z.x;
+            y += z.y;
+            nb += (!isfinite(z.x) || !isfinite(z.y)) ? 1 : 0;
+        }
+        acc[e] = m;
+        acc[cells + e] = x;
+        acc[2 * cells + e] = y;
+        if (nb) atomicAdd(bad, (double)nb);
     }
 }
 
-__global__ void k64_modes_accum(const double2* spec, long long cells, double anorm2, int first, double* acc2) {
+// acc2 (+)= sums of |a_k|^2 and |a_k|^4 over n spectra, in order.
+__global__ void k64_modes_accum(const double2* __restrict__ spec, long long cells, int n, double anorm2, int first,
+                                double* acc2) {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < cells; e += (long long)gridDim.x * blockDim.x) {
-        const double2 z = spec[e];
-        const double a2 = anorm2 * (z.x * z.x + z.y * z.y);
-        if (first) {
-            acc2[e] = a2;
-            acc2[cells + e] = a2 * a2;
-        } else {
-            acc2[e] += a2;
-            acc2[cells + e] += a2 * a2;
+        double s2 = first ? 0.0 : acc2[e], s4 = first ? 0.0 : acc2[cells + e];
+#pragma unroll 4
+        for (int s = 0; s < n; ++s) {
+            const double2 z = spec[(long long)s * cells + e];
+            const double a2 = anorm2 * (z.x * z.x + z.y * z.y);
+            s2 += a2;
+            s4 += a2 * a2;
         }
+        acc2[e] = s2;
+        acc2[cells + e] = s4;
     }
 }
 
@@ -166,64 +415,138 @@ __global__ void k64_moments_finish(const double* acc, const double* acc2, const 
     if (part_m) block_reduce_store<NP_MODES>(vm, part_m);
 }
 
-static int ew_blocks(long long n) {
+// ---------------------------------------------------------------------------------------------
+// Host side.
+namespace {
+
+int ilog2(int v) {
+    int r = 0;
+    while ((1 << r) < v) ++r;
+    return r;
+}
+int ew_blocks(long long n) {
     const long long b = (n + 255) / 256;
     return (int)(b < 152 * 16 ? b : 152 * 16);
 }
 
-int launch_f64_fft3(double2* f, const Geom64& g, const Tables64& t, bool inverse, cudaStream_t st, long long* nl) {
-    static bool big_smem = false;
-    if (!big_smem) {
-        if (cudaFuncSetAttribute(k64_fft_line, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 2048 * (int)sizeof(double2)) !=
-            cudaSuccess)
-            return -3;
-        big_smem = true;
+// Lines per CTA: 256 threads for short lines, eight lines (128 bytes of a strided access) up to 256
+// cells, then as many as 512 threads (128 registers each) hold.
+int lines64(int N) { return N <= 128 ? 1024 / N : 2048 / N; }
+
+Axis64 axis64(const Geom64& g, const Tables64& t, int a) {
+    Axis64 x{};
+    x.N = g.n[a];
+    x.lg = ilog2(x.N);
+    x.L = lines64(x.N);
+    x.S = 1;
+    for (int b = 0; b < a; ++b) x.S *= g.n[b];
+    x.cells = g.cells;
+    x.lines = g.cells / x.N;
+    x.tw = t.tw[a];
+    x.ph = t.ph[a];
+    return x;
+}
+unsigned tiles64(const Axis64& x) { return (unsigned)((x.lines + x.L - 1) / x.L); }
+int threads64(const Axis64& x) { return x.L * x.N / 4; }
+size_t smem64(const Axis64& x) { return 2 * (size_t)x.L * line64(x.N) * sizeof(double2); }
+
+// 2048 cells in a CTA: two exchange buffers of 36 KB
+int prepare64() {
+    for (const void* k : {(const void*)k64_kick_drift, (const void*)k64_drift, (const void*)k64_drift_rho,
+                          (const void*)k64_field})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
+    for (const void* k : {(const void*)k64_run1d<2>, (const void*)k64_run1d<4>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
+    return 0;
+}
+
+void field64(const Geom64& g, const Tables64& t, int a, const double2* src, double2* dst, int n, int mode, double mulc,
+             cudaStream_t st, long long* nl) {
+    const Axis64 x = axis64(g, t, a);
+    const int lx = ilog2(g.n[0]);
+    k64_field<<<dim3(tiles64(x), (unsigned)n), threads64(x), smem64(x), st>>>(x, src, dst, mode, lx, lx + ilog2(g.n[1]),
+                                                                              t.k2[0], t.k2[1], t.k2[2], mulc);
+    ++*nl;
+}
+
+// The rest of the Poisson solve of n packed fields that the last axis' forward transform begins:
+// the potentials in real space (2D), or still spectral along x (3D: the next kick undoes it).
+void poisson64(const Geom64& g, const Tables64& t, double2* W, int n, double mulc, cudaStream_t st, long long* nl) {
+    if (g.dim == 2) {
+        field64(g, t, 0, W, W, n, 2, mulc, st, nl);
+        field64(g, t, 1, W, W, n, 1, 0.0, st, nl);
+    } else {
+        field64(g, t, 0, W, W, n, 0, 0.0, st, nl);
+        field64(g, t, 1, W, W, n, 2, mulc, st, nl);
+        field64(g, t, 2, W, W, n, 1, 0.0, st, nl);
     }
-    long long stride = 1;
-    for (int a = 0; a < g.dim; ++a) {
-        const int N = g.n[a];
-        const int Qn = (int)stride;
-        const long long OS = stride * N;
-        const long long lines = g.cells / N;
-        const int thr = N / 2 < 256 ? (N / 2 > 32 ? N / 2 : 32) : 256;
-        k64_fft_line<<<(unsigned)lines, thr, 2 * N * sizeof(double2), st>>>(f, N, stride, Qn, OS, t.tw[a], inverse ? 1 : 0);
+}
+
+}  // namespace
+
+int f64_prepare() { return prepare64(); }
+
+int launch_f64_steps(double2* psi, double2* W, int w_pairs, int n_slots, const Geom64& g, const Tables64& t, double mulc,
+                     double kick, int n_steps, cudaStream_t st, long long* nl) {
+    const int last = g.dim - 1;
+    for (int s0 = 0; s0 < n_slots; s0 += 2 * w_pairs) {
+        double2* f = psi + (size_t)s0 * g.cells;
+        const int ns = n_slots - s0 < 2 * w_pairs ? n_slots - s0 : 2 * w_pairs;
+        const unsigned np = (unsigned)(ns + 1) / 2;
+        const Axis64 x0 = axis64(g, t, 0), xl = axis64(g, t, last);
+        auto rho = [&](int drift) {
+            k64_drift_rho<<<dim3(tiles64(xl), np), threads64(xl), smem64(xl), st>>>(xl, f, W, ns, drift);
+            ++*nl;
+            poisson64(g, t, W, (int)np, mulc, st, nl);
+        };
+        auto kicks = [&](double k, int drift) {
+            k64_kick_drift<<<dim3(tiles64(x0), np), threads64(x0), smem64(x0), st>>>(x0, f, W, ns, k, g.dim == 3, drift);
+            ++*nl;
+        };
+        rho(0);
+        for (int s = 0; s < n_steps; ++s) {
+            kicks(s == 0 ? 0.5 * kick : kick, 1);
+            if (g.dim == 3) {
+                const Axis64 xm = axis64(g, t, 1);
+                k64_drift<<<dim3(tiles64(xm), (unsigned)ns), threads64(xm), smem64(xm), st>>>(xm, f);
+                ++*nl;
+            }
+            rho(1);
+        }
+        kicks(0.5 * kick, 0);
+    }
+    return 0;
+}
+
+int launch_f64_run1d(double2* psi, int n_slots, const Geom64& g, const Tables64& t, double mulc, double kick, int n_out,
+                     int out_every, double* part, double* part_cl, double* part_bad, cudaStream_t st, long long* nl) {
+    const int N = g.n[0], lg = ilog2(N);
+    const size_t sm = 2 * (size_t)line64(N) * sizeof(double2);
+    if (N <= 256)
+        k64_run1d<2><<<n_slots, N / 2, sm, st>>>(psi, N, lg, t.tw[0], t.ph[0], t.k2[0], mulc, kick, n_out, out_every,
+                                                 n_slots - 1, part, part_cl, part_bad);
+    else
+        k64_run1d<4><<<n_slots, N / 4, sm, st>>>(psi, N, lg, t.tw[0], t.ph[0], t.k2[0], mulc, kick, n_out, out_every,
+                                                 n_slots - 1, part, part_cl, part_bad);
+    ++*nl;
+    return 0;
+}
+
+int launch_f64_moments_accum(const double2* psi, long long cells, int n_slots, double* acc, double* bad, cudaStream_t st,
+                             long long* nl) {
+    k64_moments_accum<<<ew_blocks(cells), 256, 0, st>>>(psi, cells, n_slots, acc, bad);
+    ++*nl;
+    return 0;
+}
+int launch_f64_modes(const double2* psi, double2* spec, int spec_fields, int n_slots, const Geom64& g, const Tables64& t,
+                     double anorm2, double* acc2, cudaStream_t st, long long* nl) {
+    for (int s = 1; s < n_slots; s += spec_fields) {
+        const int n = n_slots - s < spec_fields ? n_slots - s : spec_fields;
+        for (int a = 0; a < g.dim; ++a)
+            field64(g, t, a, a == 0 ? psi + (size_t)s * g.cells : spec, spec, n, 0, 0.0, st, nl);
+        k64_modes_accum<<<ew_blocks(g.cells), 256, 0, st>>>(spec, g.cells, n, anorm2, s == 1, acc2);
         ++*nl;
-        stride *= N;
     }
-    return 0;
-}
-int launch_f64_kinetic(double2* f, const Geom64& g, const Tables64& t, cudaStream_t st, long long* nl) {
-    G64 gg{{g.n[0], g.n[1], g.n[2]}, g.cells};
-    k64_kinetic<<<ew_blocks(g.cells), 256, 0, st>>>(f, gg, t.ph[0], t.ph[1], t.ph[2]);
-    ++*nl;
-    return 0;
-}
-int launch_f64_rho(const double2* psi, double2* work, long long cells, cudaStream_t st, long long* nl) {
-    k64_rho<<<ew_blocks(cells), 256, 0, st>>>(psi, work, cells);
-    ++*nl;
-    return 0;
-}
-int launch_f64_poisson_mul(double2* work, const Geom64& g, const Tables64& t, double mulc, cudaStream_t st, long long* nl) {
-    G64 gg{{g.n[0], g.n[1], g.n[2]}, g.cells};
-    k64_poisson_mul<<<ew_blocks(g.cells), 256, 0, st>>>(work, gg, t.k2[0], t.k2[1], t.k2[2], mulc);
-    ++*nl;
-    return 0;
-}
-int launch_f64_kick(double2* psi, const double2* work, long long cells, double kick, cudaStream_t st, long long* nl) {
-    k64_kick<<<ew_blocks(cells), 256, 0, st>>>(psi, work, cells, kick);
-    ++*nl;
-    return 0;
-}
-int launch_f64_moments_accum(const double2* psi, const double2* /*work*/, long long cells, double /*kick*/, int first,
-                             double* acc, double* bad, cudaStream_t st, long long* nl) {
-    k64_moments_accum<<<ew_blocks(cells), 256, 0, st>>>(psi, cells, first, acc, bad);
-    ++*nl;
-    return 0;
-}
-int launch_f64_modes_accum(const double2* spec, long long cells, double anorm2, int first, double* acc2, cudaStream_t st,
-                           long long* nl) {
-    k64_modes_accum<<<ew_blocks(cells), 256, 0, st>>>(spec, cells, anorm2, first, acc2);
-    ++*nl;
     return 0;
 }
 int launch_f64_moments_finish(const double* acc, const double* acc2, const double2* psi0, long long cells, int n_real,
