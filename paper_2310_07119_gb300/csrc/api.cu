@@ -904,17 +904,24 @@ int alloc_f64(twa_handle* h, Inst& I) {
     const int most = (int)std::max(1.0, std::min(32768.0, (double)(1LL << 30) / field));
     if (I.mode != MODE_1D) {
         I.w_pairs = std::min(I.n_pairs, most);
-        RC(dalloc(h, &I.work64, (size_t)I.w_pairs * I.cells));
+        while (dalloc(h, &I.work64, (size_t)I.w_pairs * I.cells) != 0) {  // fewer at a time when memory is short
+            if (I.w_pairs == 1) return TWA_ENOMEM;
+            I.w_pairs /= 2;
+        }
     } else {
         const double per_out = (double)I.n_real * (3.0 * I.cells + 1.0) + I.cells;
         I.run64_outs = (int)std::min(1024.0, (double)(16 << 20) / (8.0 * per_out)) - 1;
-        if (I.run64_outs > 0) RC(dalloc(h, &I.run64, (size_t)(I.run64_outs + 1) * (size_t)per_out));
+        // without them a 1D run takes its outputs from the moment kernels
+        if (I.run64_outs > 0 && dalloc(h, &I.run64, (size_t)(I.run64_outs + 1) * (size_t)per_out) != 0) I.run64 = nullptr;
     }
     RC(dalloc(h, &I.acc64, (size_t)3 * I.cells));
     RC(dalloc(h, &I.bad64, 1));
     if (h->p.want_modes) {
         I.spec_fields = std::min(I.n_real, most);
-        RC(dalloc(h, &I.spec64, (size_t)I.spec_fields * I.cells));
+        while (dalloc(h, &I.spec64, (size_t)I.spec_fields * I.cells) != 0) {
+            if (I.spec_fields == 1) return TWA_ENOMEM;
+            I.spec_fields /= 2;
+        }
         RC(dalloc(h, &I.acc64m, (size_t)2 * I.cells));
     }
     if (f64_prepare() != 0) return fail(h, TWA_ECUDA, "cudaFuncSetAttribute failed");

@@ -13,6 +13,7 @@
 
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "reduce.cuh"
@@ -24,143 +25,540 @@ void twa_set_global_error(const std::string& msg);
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kPwBlocks = 152 * 2;  // CTAs of the pointwise weight-gradient stage 1 (and its partials)
+constexpr int kPwBlocks = 152 * 2;  // CTAs of the pointwise weight gradient's first stage (and its partials)
+constexpr int kMixWgradSmem = 100 * 1024;
 
 int blocks_for(long long n) {
     const long long b = (n + kThreads - 1) / kThreads;
     return (int)(b < 152LL * 64 ? b : 152LL * 64);
 }
 
-__device__ __forceinline__ float bf(const __nv_bfloat16* w, long long i) { return __bfloat162float(w[i]); }
+// Packed two-lane FP32 (sm_100 and later): d = a b + c on both halves, each rounded once.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* s, const void* g) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(s)), "l"(g), "n"(BYTES));
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N)); }
 
-// Y[b][o][k] = sum_c W[o][c] X[b][c][k] + bias[o] (+ Y if accumulate); TRANS reads W as [c][o].
-template <bool TRANS>
-__global__ void k_pointwise(const float* __restrict__ X, const __nv_bfloat16* __restrict__ Wt,
-                            const float* __restrict__ bias, float* __restrict__ Y, int B, int cin, int cout,
-                            long long K, int accumulate) {
-    extern __shared__ float wsm[];
-    for (int i = threadIdx.x; i < cin * cout; i += blockDim.x) wsm[i] = __bfloat162float(Wt[i]);
-    __syncthreads();
-    const long long total = (long long)B * K;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long b = t / K, k = t - b * K;
-        float x[64];
+// out[p][i][q] = sum_j M[i][j] in[p][j][q] (complex M, nout x nin), one axis of the truncated DFT.  INR:
+// the input is real; OUTR: only the real part is kept, and added to out if accumulate.
+//
+// A batched complex matrix product with 30 to 60 FP32 operations a byte: bound by the FP32 units, once
+// their operands do not come from shared memory one by one.  A CTA owns AX_COLS columns (p, q) and up
+// to 32 outputs; a thread 8 outputs x 4 columns, two outputs to a packed FMA, so that 6 128-bit reads
+// of shared memory feed 64 packed FMAs (one thread per column and 16 outputs, an operand read per two
+// FMAs, took 5.8 ms of a 128^3 x 2 forward pass of width 32, 16 modes and 4 layers; now 1.9 ms).  The columns' values come in
+// double-buffered slices of AX_J rows by cp.async.  The sum of an output runs over j in order.
+constexpr int AX_COLS = 128, AX_J = 16, AX_O = 8;
+template <bool INR, bool OUTR>
+__global__ void __launch_bounds__(128) k_axis(const void* __restrict__ in, const float2* __restrict__ M, void* __restrict__ out,
+                                              long long cols, int nin, int nout, long long Q, int accumulate) {
+    extern __shared__ __align__(16) float4 axsm[];
+    using X = typename std::conditional<INR, float, float2>::type;
+    const int og = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ob = blockIdx.y * 4 * AX_O, o0 = ob + og * AX_O;   // this CTA's and this warp's outputs
+    float4* Ms = axsm;                                          // [j][pair of outputs] (re0, re1, im0, im1)
+    X* Xs = reinterpret_cast<X*>(Ms + (size_t)2 * AX_O * nin);  // [2][AX_J][AX_COLS]
+    for (int t = threadIdx.x; t < 2 * AX_O * nin; t += 128) {
+        const int pr = t / nin, j = t - pr * nin, i = ob + 2 * pr;
+        const float2 a = i < nout ? M[(long long)i * nin + j] : make_float2(0.f, 0.f);
+        const float2 b = i + 1 < nout ? M[(long long)(i + 1) * nin + j] : make_float2(0.f, 0.f);
+        Ms[j * 2 * AX_O + pr] = make_float4(a.x, b.x, a.y, b.y);
+    }
+    const long long c0 = (long long)blockIdx.x * AX_COLS;
+    // copies: a thread per column where those are contiguous, lanes along j where the axis is (Q = 1)
+    const X* src = static_cast<const X*>(in);
+    {
+        const long long col = min(c0 + threadIdx.x, cols - 1), p = Q == 1 ? 0 : col / Q;
+        if (Q != 1) src += p * nin * Q + (col - p * Q);
+    }
+    auto load = [&](int j0, int buf) {
+        X* dst = Xs + buf * AX_J * AX_COLS;
+        if (Q != 1) {
+#pragma unroll
+            for (int jj = 0; jj < AX_J; ++jj)
+                if (j0 + jj < nin) cp_async<sizeof(X)>(dst + jj * AX_COLS + threadIdx.x, src + (long long)(j0 + jj) * Q);
+        } else {
+            const int jj = threadIdx.x % AX_J;
 #pragma unroll 4
-        for (int c = 0; c < cin; ++c) x[c] = X[(b * cin + c) * K + k];
-        for (int o = 0; o < cout; ++o) {
-            float acc = bias ? bias[o] : 0.f;
-            for (int c = 0; c < cin; ++c) acc = fmaf(TRANS ? wsm[c * cout + o] : wsm[o * cin + c], x[c], acc);
-            float* y = &Y[(b * cout + o) * K + k];
-            *y = accumulate ? *y + acc : acc;
+            for (int c = threadIdx.x / AX_J; c < AX_COLS; c += 128 / AX_J)
+                if (j0 + jj < nin)
+                    cp_async<sizeof(X)>(dst + jj * AX_COLS + c, src + min(c0 + c, cols - 1) * nin + j0 + jj);
         }
-    }
-}
-
-// Stage 1 of dW[o][c] = sum_{b,k} dY[b][o][k] X[b][c][k] and db[o] = sum dY: block (o, chunk) sums a
-// fixed chunk of positions; stage 2 adds the chunks in order.
-__global__ void k_pointwise_wgrad_part(const float* __restrict__ dY, const float* __restrict__ X, int B, int cin,
-                                       int cout, long long K, int nchunk, float* __restrict__ part) {
-    const int o = blockIdx.x, ch = blockIdx.y;
-    const long long total = (long long)B * K;
-    const long long per = (total + nchunk - 1) / nchunk;
-    const long long lo = ch * per, hi = (lo + per < total) ? lo + per : total;
-    float acc[65];
-    for (int c = 0; c <= cin; ++c) acc[c] = 0.f;
-    for (long long t = lo + threadIdx.x; t < hi; t += blockDim.x) {
-        const long long b = t / K, k = t - b * K;
-        const float g = dY[(b * cout + o) * K + k];
-        for (int c = 0; c < cin; ++c) acc[c] = fmaf(g, X[(b * cin + c) * K + k], acc[c]);
-        acc[cin] += g;
-    }
-    __shared__ float red[kThreads];
-    for (int c = 0; c <= cin; ++c) {
-        red[threadIdx.x] = acc[c];
-        __syncthreads();
-        for (int s = kThreads / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-            __syncthreads();
+        cp_commit();
+    };
+    float2 ar[AX_O / 2][4], ai[AX_O / 2][4];
+#pragma unroll
+    for (int u = 0; u < AX_O / 2; ++u)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ar[u][c] = ai[u][c] = make_float2(0.f, 0.f);
+    const int slices = (nin + AX_J - 1) / AX_J;
+    load(0, 0);
+    for (int s = 0; s < slices; ++s) {
+        if (s + 1 < slices) {
+            load((s + 1) * AX_J, (s + 1) & 1);
+            cp_wait<1>();
+        } else {
+            cp_wait<0>();
         }
-        if (threadIdx.x == 0) part[((long long)o * nchunk + ch) * (cin + 1) + c] = red[0];
         __syncthreads();
-    }
-}
-
-__global__ void k_pointwise_wgrad_sum(const float* __restrict__ part, int cin, int cout, int nchunk,
-                                      float* __restrict__ dW, float* __restrict__ db) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cout * (cin + 1)) return;
-    const int o = i / (cin + 1), c = i % (cin + 1);
-    float s = 0.f;
-    for (int ch = 0; ch < nchunk; ++ch) s += part[((long long)o * nchunk + ch) * (cin + 1) + c];
-    if (c < cin) dW[o * cin + c] += s;
-    else db[o] += s;
-}
-
-// out[p][i][q] = sum_j M[i][j] in[p][j][q] (complex M, nout x nin); in may be real; out may keep the
-// real part only (then optionally added to out).
-__global__ void k_axis(const float2* __restrict__ in_c, const float* __restrict__ in_r, const float2* __restrict__ M,
-                       float2* __restrict__ out_c, float* __restrict__ out_r, long long P, int nin, int nout,
-                       long long Q, int accumulate) {
-    const long long total = P * nout * Q;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long q = t % Q;
-        const long long r = t / Q;
-        const int i = (int)(r % nout);
-        const long long p = r / nout;
-        float ar = 0.f, ai = 0.f;
-        for (int j = 0; j < nin; ++j) {
-            const float2 m = M[i * nin + j];
-            const long long src = (p * nin + j) * Q + q;
-            if (in_r) {
-                const float x = in_r[src];
-                ar = fmaf(m.x, x, ar);
-                ai = fmaf(m.y, x, ai);
+        const X* xs = Xs + (size_t)(s & 1) * AX_J * AX_COLS + lane * 4;
+        const int nj = min(AX_J, nin - s * AX_J);
+        if (o0 < nout)
+#pragma unroll 4
+        for (int jj = 0; jj < nj; ++jj) {
+            const float4* m = Ms + (s * AX_J + jj) * 2 * AX_O + og * (AX_O / 2);
+            float2 x[4];
+            if constexpr (INR) {
+                const float4 v = *reinterpret_cast<const float4*>(xs + jj * AX_COLS);
+                x[0].x = v.x;
+                x[1].x = v.y;
+                x[2].x = v.z;
+                x[3].x = v.w;
             } else {
-                const float2 x = in_c[src];
-                ar = fmaf(m.x, x.x, fmaf(-m.y, x.y, ar));
-                ai = fmaf(m.x, x.y, fmaf(m.y, x.x, ai));
+                const float4 v = reinterpret_cast<const float4*>(xs + jj * AX_COLS)[0];
+                const float4 w = reinterpret_cast<const float4*>(xs + jj * AX_COLS)[1];
+                x[0] = make_float2(v.x, v.y);
+                x[1] = make_float2(v.z, v.w);
+                x[2] = make_float2(w.x, w.y);
+                x[3] = make_float2(w.z, w.w);
+            }
+#pragma unroll
+            for (int u = 0; u < AX_O / 2; ++u) {
+                const float4 mm = m[u];
+                const float2 mr = make_float2(mm.x, mm.y), mi = make_float2(mm.z, mm.w);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float2 xr = make_float2(x[c].x, x[c].x);
+                    if constexpr (INR) {
+                        ar[u][c] = fma2(mr, xr, ar[u][c]);
+                        ai[u][c] = fma2(mi, xr, ai[u][c]);
+                    } else {
+                        const float2 xn = make_float2(-x[c].y, -x[c].y), xi = make_float2(x[c].y, x[c].y);
+                        ar[u][c] = fma2(mr, xr, fma2(mi, xn, ar[u][c]));
+                        if constexpr (!OUTR) ai[u][c] = fma2(mr, xi, fma2(mi, xr, ai[u][c]));
+                    }
+                }
             }
         }
-        if (out_r) out_r[t] = accumulate ? out_r[t] + ar : ar;
-        else out_c[t] = make_float2(ar, ai);
+        __syncthreads();
     }
-}
-
-// Ymix[b][o][m] = sum_c R[m][o][c] S[b][c][m]  (R complex, BF16 re/im); ADJ: dS[b][c][m] = sum_o conj(R[m][o][c]) G[b][o][m]
-template <bool ADJ>
-__global__ void k_mix(const float2* __restrict__ S, const __nv_bfloat16* __restrict__ R, float2* __restrict__ Y, int B,
-                      int W, long long Mm) {
-    const long long total = (long long)B * W * Mm;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long m = t % Mm;
-        const long long r = t / Mm;
-        const int o = (int)(r % W);
-        const long long b = r / W;
-        float ar = 0.f, ai = 0.f;
-        for (int c = 0; c < W; ++c) {
-            const long long ri = ADJ ? ((m * W + c) * W + o) * 2 : ((m * W + o) * W + c) * 2;
-            const float rr = bf(R, ri), rim = ADJ ? -bf(R, ri + 1) : bf(R, ri + 1);
-            const float2 x = S[(b * W + c) * Mm + m];
-            ar = fmaf(rr, x.x, fmaf(-rim, x.y, ar));
-            ai = fmaf(rr, x.y, fmaf(rim, x.x, ai));
+    if (o0 >= nout) return;
+    const long long col = c0 + lane * 4;
+    if (!OUTR && (Q & 3) == 0) {  // the four columns are neighbours in memory
+        if (col >= cols) return;
+        const long long p = col / Q, q = col - p * Q;
+#pragma unroll
+        for (int u = 0; u < AX_O; ++u) {
+            if (o0 + u >= nout) break;
+            float4* d = reinterpret_cast<float4*>(static_cast<float2*>(out) + (p * nout + o0 + u) * Q + q);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                d[h] = u & 1 ? make_float4(ar[u / 2][2 * h].y, ai[u / 2][2 * h].y, ar[u / 2][2 * h + 1].y, ai[u / 2][2 * h + 1].y)
+                             : make_float4(ar[u / 2][2 * h].x, ai[u / 2][2 * h].x, ar[u / 2][2 * h + 1].x, ai[u / 2][2 * h + 1].x);
         }
-        Y[t] = make_float2(ar, ai);
+        return;
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        if (col + c >= cols) break;
+        const long long p = Q == 1 ? col + c : (col + c) / Q, q = col + c - p * Q;
+#pragma unroll
+        for (int u = 0; u < AX_O; ++u) {
+            const int i = o0 + u;
+            if (i >= nout) break;
+            const long long d = (p * nout + i) * Q + q;
+            const float re = u & 1 ? ar[u / 2][c].y : ar[u / 2][c].x;
+            if constexpr (OUTR) {
+                float* o = static_cast<float*>(out);
+                o[d] = accumulate ? o[d] + re : re;
+            } else {
+                static_cast<float2*>(out)[d] = make_float2(re, u & 1 ? ai[u / 2][c].y : ai[u / 2][c].x);
+            }
+        }
     }
 }
 
-// dR[m][o][c] += sum_b G[b][o][m] conj(S[b][c][m])   (re/im interleaved in the flat gradient)
-__global__ void k_mix_wgrad(const float2* __restrict__ G, const float2* __restrict__ S, float* __restrict__ dR, int B,
-                            int W, long long Mm) {
+__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
+__device__ __forceinline__ float gelu_g(float z) {
+    return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
+}
+
+// Y[b][o][k] = sum_c W[o][c] X[b][c][k] + bias[o] (+ Y if accumulate); TRANS reads W as [c][o].  What
+// follows the map in the network is part of it: EP_GELU also stores gelu(Y) to Z, EP_GRAD stores
+// Y gelu'(Z) instead of Y.
+//
+// Bound by memory (width 32 with EP_GELU: 4 arrays of 128 bytes a position for 1024 FMAs) as long as
+// the weights are cheap and enough loads are in flight: a thread holds PW_O outputs of P positions, two
+// outputs to a packed FMA, so that a 128-bit read of the weights feeds 2 P of them, eight inputs ahead.
+// 32 outputs take two positions: four need 220 registers and leave 8 warps an SM.
+// Positions come P to a load when every row starts on 16 bytes (VEC), else one by one, a block apart.  (One position per thread, its inputs
+// in local memory, and gelu passes of their own took 5.1 ms of a 128^3 x 2 forward pass; now 2.5 ms.)
+enum { EP_NONE = 0, EP_GELU, EP_GRAD };
+template <int PW_O, int P, bool TRANS, int EP, bool VEC>
+__global__ void __launch_bounds__(128, 4) k_pointwise(const float* __restrict__ X, const __nv_bfloat16* __restrict__ Wt,
+                                                   const float* __restrict__ bias, float* Y, float* Z, int B, int cin,
+                                                   int cout, long long K, int accumulate) {
+    __shared__ __align__(16) float ws[64 * PW_O];   // [c][o] of this block of outputs
+    __shared__ float bs[PW_O];
+    const int o0 = blockIdx.y * PW_O;
+    for (int i = threadIdx.x; i < cin * PW_O; i += 128) {
+        const int c = i / PW_O, o = o0 + i % PW_O;
+        ws[i] = o < cout ? __bfloat162float(Wt[TRANS ? c * cout + o : o * cin + c]) : 0.f;
+    }
+    for (int i = threadIdx.x; i < PW_O; i += 128) bs[i] = bias && o0 + i < cout ? bias[o0 + i] : 0.f;
+    __syncthreads();
+    // positions k0 + u st, u < P
+    const long long k0 = blockIdx.x * (128LL * P) + threadIdx.x * (VEC ? P : 1);
+    const int st = VEC ? 1 : 128;
+    if (k0 >= K) return;
+    auto get = [&](const float* p, float (&v)[P]) {
+        if constexpr (VEC && P == 4) {
+            const float4 t = *reinterpret_cast<const float4*>(p);
+            v[0] = t.x;
+            v[1] = t.y;
+            v[2] = t.z;
+            v[3] = t.w;
+        } else if constexpr (VEC) {
+            const float2 t = *reinterpret_cast<const float2*>(p);
+            v[0] = t.x;
+            v[1] = t.y;
+        } else {
+#pragma unroll
+            for (int u = 0; u < P; ++u) v[u] = k0 + u * st < K ? p[u * st] : 0.f;
+        }
+    };
+    auto put = [&](float* p, const float (&v)[P]) {
+        if constexpr (VEC && P == 4) {
+            *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+        } else if constexpr (VEC) {
+            *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < P; ++u)
+                if (k0 + u * st < K) p[u * st] = v[u];
+        }
+    };
+    for (long long b = blockIdx.z; b < B; b += gridDim.z) {
+        const float* x = X + b * cin * K + k0;
+        float2 acc[PW_O / 2][P];
+#pragma unroll
+        for (int o = 0; o < PW_O / 2; ++o)
+#pragma unroll
+            for (int u = 0; u < P; ++u) acc[o][u] = make_float2(bs[2 * o], bs[2 * o + 1]);
+#pragma unroll 8
+        for (int c = 0; c < cin; ++c) {
+            float v[P];
+            get(x + c * K, v);
+            const float4* w = reinterpret_cast<const float4*>(ws + c * PW_O);
+#pragma unroll
+            for (int o = 0; o < PW_O / 4; ++o) {
+                const float4 ww = w[o];
+#pragma unroll
+                for (int u = 0; u < P; ++u) {
+                    acc[2 * o][u] = fma2(make_float2(ww.x, ww.y), make_float2(v[u], v[u]), acc[2 * o][u]);
+                    acc[2 * o + 1][u] = fma2(make_float2(ww.z, ww.w), make_float2(v[u], v[u]), acc[2 * o + 1][u]);
+                }
+            }
+        }
+        // G outputs at a time: their loads first, as the stores may alias them for the compiler
+        constexpr int G = PW_O < 8 ? PW_O : 8;
+#pragma unroll
+        for (int og = 0; og < PW_O; og += G) {
+            if (o0 + og >= cout) break;
+            float t[G][P], z[G][P];
+            const long long at = (b * cout + o0 + og) * K + k0;
+#pragma unroll
+            for (int o = 0; o < G; ++o)
+                if (accumulate && o0 + og + o < cout) get(Y + at + o * K, t[o]);
+            if constexpr (EP == EP_GRAD) {
+#pragma unroll
+                for (int o = 0; o < G; ++o)
+                    if (o0 + og + o < cout) get(Z + at + o * K, z[o]);
+            }
+#pragma unroll
+            for (int o = 0; o < G; ++o) {
+                if (o0 + og + o >= cout) break;
+                float r[P];
+#pragma unroll
+                for (int u = 0; u < P; ++u) {
+                    r[u] = (og + o) & 1 ? acc[(og + o) / 2][u].y : acc[(og + o) / 2][u].x;
+                    if (accumulate) r[u] = t[o][u] + r[u];
+                    if constexpr (EP == EP_GRAD) r[u] = r[u] * gelu_g(z[o][u]);
+                }
+                put(Y + at + o * K, r);
+                if constexpr (EP == EP_GELU) {
+#pragma unroll
+                    for (int u = 0; u < P; ++u) r[u] = gelu_f(r[u]);
+                    put(Z + at + o * K, r);
+                }
+            }
+        }
+    }
+}
+
+// Partial sums of dW[o][c] = sum_{b,k} dY[b][o][k] X[b][c][k] and db[o] = sum dY over the chunks of
+// positions of CTA blockIdx.x, for outputs and inputs in blocks of 32 (blockIdx.y).  part[o][blk][c],
+// c = cin for db; k_pointwise_wgrad_sum adds the blocks in a fixed order.
+//
+// The 32 x 32 sums sit in the registers of 16 threads (8 x 8 each), and 16 such groups take every
+// sixteenth group of four positions of a chunk, copied to shared memory one chunk ahead: 16 128-bit
+// reads feed 256 FMAs (one product per two reads took 536 us a call at 64^3 x 4, width 32, 24 times its reads from HBM;
+// now 90 us).  Rows are padded so that the eight rows a quarter warp reads lie in distinct banks.
+constexpr int WG_CH = 128, WG_LD = WG_CH + 4, WG_SMEM = 2 * 64 * WG_LD * 4;
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_pointwise_wgrad(const float* __restrict__ dY, const float* __restrict__ X, int B,
+                                                         int cin, int cout, long long K, float* __restrict__ part) {
+    extern __shared__ __align__(16) float wgsm[];     // two buffers of 32 rows of dY, 32 rows of X
+    __shared__ float sb[16][32];
+    const int nci = (cin + 31) / 32, o0 = (blockIdx.y / nci) * 32, i0 = (blockIdx.y % nci) * 32;
+    const int grp = threadIdx.x / 16, ty = (threadIdx.x % 16) / 4, tx = threadIdx.x % 4;  // rows ty + 4 u, tx + 4 u
+    float acc[8][8], ab[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        ab[u] = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) acc[u][w] = 0.f;
+    }
+    const long long kch = (K + WG_CH - 1) / WG_CH, total = (long long)B * kch;
+    // rows past the last output or input stay zero; positions past the last are copied as zeros
+    for (int i = threadIdx.x; i < 2 * 64 * WG_LD; i += 256) wgsm[i] = 0.f;
+    __syncthreads();
+    auto load = [&](long long ch, float* dst) {
+        const long long b = ch / kch, k0 = (ch - b * kch) * WG_CH;
+        constexpr int E = VEC ? 4 : 1, PER = WG_CH / E;   // floats per copy, copies per row
+#pragma unroll 8
+        for (int i = threadIdx.x; i < 64 * PER; i += 256) {
+            const int row = i / PER, k = (i % PER) * E;
+            const bool y = row < 32;
+            const int r = y ? o0 + row : i0 + row - 32;
+            if (r >= (y ? cout : cin)) continue;
+            const bool in = k0 + k < K;
+            const float* g = (y ? dY : X) + (b * (y ? cout : cin) + r) * K + (in ? k0 + k : 0);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((unsigned)__cvta_generic_to_shared(dst + row * WG_LD + k)),
+                         "l"(g), "n"(E * 4), "r"(in ? E * 4 : 0));
+        }
+        cp_commit();
+    };
+    if (blockIdx.x < total) load(blockIdx.x, wgsm);
+    int buf = 0;
+    for (long long ch = blockIdx.x; ch < total; ch += gridDim.x, buf ^= 1) {
+        if (ch + gridDim.x < total) {
+            load(ch + gridDim.x, wgsm + (buf ^ 1) * 64 * WG_LD);
+            cp_wait<1>();
+        } else {
+            cp_wait<0>();
+        }
+        __syncthreads();
+        const float* cur = wgsm + buf * 64 * WG_LD;
+#pragma unroll
+        for (int g = 0; g < WG_CH / 64; ++g) {
+            const float* s = cur + (grp + 16 * g) * 4;
+            float4 y[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                y[u] = *reinterpret_cast<const float4*>(s + (ty + 4 * u) * WG_LD);
+                if (tx == 0) ab[u] += (y[u].x + y[u].y) + (y[u].z + y[u].w);
+            }
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                const float4 x = *reinterpret_cast<const float4*>(s + (32 + tx + 4 * w) * WG_LD);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    acc[u][w] = fmaf(y[u].w, x.w, fmaf(y[u].z, x.z, fmaf(y[u].y, x.y, fmaf(y[u].x, x.x, acc[u][w]))));
+            }
+        }
+        __syncthreads();
+    }
+    // the sixteen groups' sums in group order, four rows u at a time (16 x 4 x 32 floats each)
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (tx == 0) sb[grp][ty + 4 * u] = ab[u];
+    const int nb = gridDim.x;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int w = 0; w < 8; ++w) wgsm[(grp * 16 + ty + 4 * u) * 32 + tx + 4 * w] = acc[4 * h + u][w];
+        __syncthreads();
+        for (int t = threadIdx.x; t < 512; t += 256) {
+            float v = 0.f;
+#pragma unroll
+            for (int g = 0; g < 16; ++g) v += wgsm[g * 512 + t];
+            const int o = o0 + 16 * h + t / 32, c = i0 + t % 32;
+            if (o < cout && c < cin) part[((long long)o * nb + blockIdx.x) * (cin + 1) + c] = v;
+        }
+    }
+    if (i0 == 0 && threadIdx.x < 32 && o0 + threadIdx.x < cout) {
+        float v = 0.f;
+#pragma unroll
+        for (int g = 0; g < 16; ++g) v += sb[g][threadIdx.x];
+        part[((long long)(o0 + threadIdx.x) * nb + blockIdx.x) * (cin + 1) + cin] = v;
+    }
+}
+
+// dW and db += the blocks' partial sums: a CTA of 128 threads per output o; thread t adds blocks in
+// order for its c (a tree over a warp's lanes would read them uncoalesced).
+__global__ void k_pointwise_wgrad_sum(const float* __restrict__ part, int cin, int nblk, float* __restrict__ dW,
+                                      float* __restrict__ db) {
+    // 128 threads: (cin + 1) columns in up to 128 / (cin + 1) slices of the blocks, the slices added in order
+    __shared__ float red[128];
+    const int o = blockIdx.x, nc = cin + 1, slices = 128 / nc, sl = threadIdx.x / nc, c = threadIdx.x % nc;
+    float s = 0.f;
+    if (sl < slices)
+        for (int i = sl; i < nblk; i += slices) s += part[((long long)o * nblk + i) * nc + c];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (sl == 0) {
+        for (int u = 1; u < slices; ++u) s += red[u * nc + c];
+        if (c < cin) dW[o * cin + c] += s;
+        else db[o] += s;
+    }
+}
+
+// Per retained mode m: Y[b][o] = sum_c R[o][c] S[b][c], or ADJ: dS[b][c] = sum_o conj(R[o][c]) G[b][o] (R
+// complex BF16, W x W).  Every R is used once, so the call is bound by reading R (134 MB at 32^3 modes
+// and width 32): thread (x, mode) holds one output channel x for MIX_B batch elements, reads its row
+// of R four complex numbers at a time (R4; rows of an ADJ product are read across the threads), and
+// takes the modes' inputs from shared memory, where a warp's threads read one address.  CTAs of
+// MIX_T / W modes.  (R staged in shared memory and read with a 16-way bank conflict, in two CTAs per
+// SM, took 356 us a call at 128^3 x 2; now 58 us.)
+constexpr int MIX_T = 256, MIX_B = 4;
+enum { R_SCALAR = 0, R_COMPLEX, R_FOUR };   // loads of R: its reals, complex numbers, four of them
+template <bool ADJ, int RL>
+__global__ void __launch_bounds__(MIX_T) k_mix(const float2* __restrict__ S, const __nv_bfloat16* __restrict__ R,
+                                               float2* __restrict__ Y, int B, int W, long long Mm, int MB) {
+    extern __shared__ float2 mxsm[];
+    const int LD = W + 1;                             // padded: the copies walk along the modes
+    float2* Ss = mxsm;                                // [min(B, MIX_B)][mode][W]
+    float2* Ys = Ss + (size_t)MIX_B * MB * LD;        // the same of the results
+    const int x = threadIdx.x % W, mm = threadIdx.x / W, nt = MB * W;
+    const long long m0 = (long long)blockIdx.x * MB;
+    const int nm = (int)min((long long)MB, Mm - m0);
+    for (int b0 = 0; b0 < B; b0 += MIX_B) {
+        const int nb = min(MIX_B, B - b0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < nb * W * MB; i += nt) {
+            const int k = i % MB, bc = i / MB;
+            if (k < nm) Ss[((bc / W) * MB + k) * LD + bc % W] = S[((long long)b0 * W + bc) * Mm + m0 + k];
+        }
+        __syncthreads();
+        if (mm < nm) {
+            float2 acc[MIX_B];
+#pragma unroll
+            for (int b = 0; b < MIX_B; ++b) acc[b] = make_float2(0.f, 0.f);
+            const long long r0 = (m0 + mm) * W * W + (ADJ ? x : (long long)x * W);   // complex elements
+            auto step = [&](int c, __nv_bfloat162 q) {
+                const float2 w = __bfloat1622float2(q);
+                const float rim = ADJ ? -w.y : w.y;
+#pragma unroll
+                for (int b = 0; b < MIX_B; ++b) {
+                    if (b >= nb) break;
+                    const float2 v = Ss[(b * MB + mm) * LD + c];
+                    acc[b].x = fmaf(w.x, v.x, fmaf(-rim, v.y, acc[b].x));
+                    acc[b].y = fmaf(w.x, v.y, fmaf(rim, v.x, acc[b].y));
+                }
+            };
+            if constexpr (RL == R_FOUR) {
+                const uint4* r = reinterpret_cast<const uint4*>(R + 2 * r0);
+#pragma unroll 4
+                for (int c = 0; c < W; c += 4) {
+                    const uint4 q = r[c / 4];
+                    step(c, *reinterpret_cast<const __nv_bfloat162*>(&q.x));
+                    step(c + 1, *reinterpret_cast<const __nv_bfloat162*>(&q.y));
+                    step(c + 2, *reinterpret_cast<const __nv_bfloat162*>(&q.z));
+                    step(c + 3, *reinterpret_cast<const __nv_bfloat162*>(&q.w));
+                }
+            } else {
+#pragma unroll 8
+                for (int c = 0; c < W; ++c) {
+                    const long long d = r0 + (ADJ ? (long long)c * W : c);
+                    step(c, RL == R_COMPLEX ? reinterpret_cast<const __nv_bfloat162*>(R)[d]
+                                            : __nv_bfloat162(R[2 * d], R[2 * d + 1]));
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < MIX_B; ++b)
+                if (b < nb) Ys[(b * MB + mm) * LD + x] = acc[b];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nb * W * MB; i += nt) {
+            const int k = i % MB, bc = i / MB;
+            if (k < nm) Y[((long long)b0 * W + bc) * Mm + m0 + k] = Ys[((bc / W) * MB + k) * LD + bc % W];
+        }
+    }
+}
+
+// dR[m][o][c] += sum_b G[b][o][m] conj(S[b][c][m])   (re/im interleaved in the flat gradient): bound by
+// reading and writing dR (2 x 268 MB at 32^3 modes and width 32).  A CTA holds the inputs of MB modes
+// in shared memory with the channels side by side, so that threads on consecutive c read distinct
+// banks (PAIR: two c and 16 bytes of dR per thread).  With the modes side by side it took 316 us a
+// call at 64^3 x 4, width 32, 32^3 modes; now 126 us.
+template <bool PAIR>
+__global__ void __launch_bounds__(MIX_T) k_mix_wgrad(const float2* __restrict__ G, const float2* __restrict__ S,
+                                                     float* __restrict__ dR, int B, int W, long long Mm, int MB) {
+    extern __shared__ float2 mxsm[];
+    const int LD = W + 1;
+    float2* Gs = mxsm;                       // [B][mode][W]
+    float2* Ss = Gs + (size_t)B * MB * LD;
+    const long long m0 = (long long)blockIdx.x * MB;
+    const int nm = (int)min((long long)MB, Mm - m0);
+    for (int i = threadIdx.x; i < B * W * MB; i += MIX_T) {
+        const int k = i % MB, bc = i / MB;
+        if (k < nm) {
+            Gs[((bc / W) * MB + k) * LD + bc % W] = G[(long long)bc * Mm + m0 + k];
+            Ss[((bc / W) * MB + k) * LD + bc % W] = S[(long long)bc * Mm + m0 + k];
+        }
+    }
+    __syncthreads();
+    auto dot = [&](int mm, int o, int c) {
+        float2 a = make_float2(0.f, 0.f);
+        for (int b = 0; b < B; ++b) {
+            const float2 g = Gs[(b * MB + mm) * LD + o], v = Ss[(b * MB + mm) * LD + c];
+            a.x = fmaf(g.x, v.x, fmaf(g.y, v.y, a.x));
+            a.y = fmaf(g.y, v.x, fmaf(-g.x, v.y, a.y));
+        }
+        return a;
+    };
+    if constexpr (PAIR) {
+        float4* d = reinterpret_cast<float4*>(dR + 2 * m0 * W * W);
+        const int h = W / 2;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < nm * W * h; i += MIX_T) {
+            const int c = i % h, o = (i / h) % W, mm = i / (h * W);
+            const float2 p = dot(mm, o, 2 * c), q = dot(mm, o, 2 * c + 1);
+            const float4 r = d[i];
+            d[i] = make_float4(r.x + p.x, r.y + p.y, r.z + q.x, r.w + q.y);
+        }
+    } else {
+        for (int i = threadIdx.x; i < nm * W * W; i += MIX_T) {
+            const float2 p = dot(i / (W * W), (i / W) % W, i % W);
+            const long long t = m0 * W * W + i;
+            dR[2 * t] += p.x;
+            dR[2 * t + 1] += p.y;
+        }
+    }
+}
+
+// The same without shared memory, for batches whose inputs of one mode exceed it.
+__global__ void k_mix_wgrad_any(const float2* __restrict__ G, const float2* __restrict__ S, float* __restrict__ dR, int B,
+                                int W, long long Mm) {
     const long long total = Mm * W * W;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(t % W);
-        const long long r = t / W;
-        const int o = (int)(r % W);
-        const long long m = r / W;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
+        const int c = (int)(t % W), o = (int)((t / W) % W);
+        const long long m = t / ((long long)W * W);
         float ar = 0.f, ai = 0.f;
         for (int b = 0; b < B; ++b) {
             const float2 g = G[((long long)b * W + o) * Mm + m];
@@ -171,200 +569,6 @@ __global__ void k_mix_wgrad(const float2* __restrict__ G, const float2* __restri
         dR[2 * t] += ar;
         dR[2 * t + 1] += ai;
     }
-}
-
-// ---------------------------------------------------------------------------------------------
-// Restructured contractions (same sums, same order per output; fewer passes over the inputs).
-
-// out[p][i][q] = sum_j M[i][j] in[p][j][q] (as k_axis): one thread per (p, q) and group of up to AG
-// outputs i, so every input value is read once per group; M is staged in shared memory and read
-// by the whole warp at the same address.
-constexpr int AG = 16;
-__global__ void k_axis_g(const float2* __restrict__ in_c, const float* __restrict__ in_r, const float2* __restrict__ M,
-                         float2* __restrict__ out_c, float* __restrict__ out_r, long long P, int nin, int nout, long long Q,
-                         int accumulate) {
-    extern __shared__ float2 Ms[];
-    for (int i = threadIdx.x; i < nin * nout; i += blockDim.x) Ms[i] = M[i];
-    __syncthreads();
-    const int ng = (nout + AG - 1) / AG;
-    const long long total = P * ng * Q;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long q = t % Q;
-        const long long r = t / Q;
-        const int g = (int)(r % ng);
-        const long long p = r / ng;
-        const int i0 = g * AG;
-        float ar[AG], ai[AG];
-#pragma unroll
-        for (int u = 0; u < AG; ++u) ar[u] = ai[u] = 0.f;
-        for (int j = 0; j < nin; ++j) {
-            const long long src = (p * nin + j) * Q + q;
-            if (in_r) {
-                const float x = in_r[src];
-#pragma unroll
-                for (int u = 0; u < AG; ++u) {
-                    const float2 m = Ms[min(i0 + u, nout - 1) * nin + j];
-                    ar[u] = fmaf(m.x, x, ar[u]);
-                    ai[u] = fmaf(m.y, x, ai[u]);
-                }
-            } else {
-                const float2 x = in_c[src];
-#pragma unroll
-                for (int u = 0; u < AG; ++u) {
-                    const float2 m = Ms[min(i0 + u, nout - 1) * nin + j];
-                    ar[u] = fmaf(m.x, x.x, fmaf(-m.y, x.y, ar[u]));
-                    ai[u] = fmaf(m.x, x.y, fmaf(m.y, x.x, ai[u]));
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < AG; ++u) {
-            const int i = i0 + u;
-            if (i >= nout) break;
-            const long long dst = (p * nout + i) * Q + q;
-            if (out_r) out_r[dst] = accumulate ? out_r[dst] + ar[u] : ar[u];
-            else out_c[dst] = make_float2(ar[u], ai[u]);
-        }
-    }
-}
-
-// k_mix with a CTA per block of MB modes: the modes' R matrices (W x W complex BF16) and the inputs
-// of every batch element for them are staged in shared memory, so R is read from memory once per
-// call instead of once per batch element.  Thread (x, mm): x = output channel (o, or c for ADJ).
-template <bool ADJ>
-__global__ void k_mix_g(const float2* __restrict__ S, const __nv_bfloat16* __restrict__ R, float2* __restrict__ Y, int B,
-                        int W, long long Mm, int MB) {
-    extern __shared__ float2 sm[];
-    float2* Rs = sm;                              // [MB][W][W]
-    float2* Ss = sm + (size_t)MB * W * W;         // [B][W][MB]
-    const int x = threadIdx.x % W, mm = threadIdx.x / W;
-    for (long long m0 = (long long)blockIdx.x * MB; m0 < Mm; m0 += (long long)gridDim.x * MB) {
-        const int nm = (int)min((long long)MB, Mm - m0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < nm * W * W; i += blockDim.x) {
-            const long long ri = (m0 * W * W + i) * 2;
-            Rs[i] = make_float2(bf(R, ri), bf(R, ri + 1));
-        }
-        for (int i = threadIdx.x; i < B * W * MB; i += blockDim.x) {
-            const int k = i % MB, bc = i / MB;
-            Ss[i] = (k < nm) ? S[(long long)bc * Mm + m0 + k] : make_float2(0.f, 0.f);
-        }
-        __syncthreads();
-        if (mm < nm) {
-            for (int b = 0; b < B; ++b) {
-                float ar = 0.f, ai = 0.f;
-                for (int c = 0; c < W; ++c) {
-                    const float2 r = ADJ ? Rs[((size_t)mm * W + c) * W + x] : Rs[((size_t)mm * W + x) * W + c];
-                    const float rim = ADJ ? -r.y : r.y;
-                    const float2 v = Ss[((size_t)b * W + c) * MB + mm];
-                    ar = fmaf(r.x, v.x, fmaf(-rim, v.y, ar));
-                    ai = fmaf(r.x, v.y, fmaf(rim, v.x, ai));
-                }
-                Y[((long long)b * W + x) * Mm + m0 + mm] = make_float2(ar, ai);
-            }
-        }
-    }
-}
-
-// k_mix_wgrad with a CTA per block of MB modes: G and S of those modes staged in shared memory, one
-// thread per (o, c) pair of a mode, writes consecutive in c.
-__global__ void k_mix_wgrad_g(const float2* __restrict__ G, const float2* __restrict__ S, float* __restrict__ dR, int B,
-                              int W, long long Mm, int MB) {
-    extern __shared__ float2 sm[];
-    float2* Gs = sm;                         // [B][W][MB]
-    float2* Ss = sm + (size_t)B * W * MB;    // [B][W][MB]
-    for (long long m0 = (long long)blockIdx.x * MB; m0 < Mm; m0 += (long long)gridDim.x * MB) {
-        const int nm = (int)min((long long)MB, Mm - m0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < B * W * MB; i += blockDim.x) {
-            const int k = i % MB, bc = i / MB;
-            const bool in = k < nm;
-            Gs[i] = in ? G[(long long)bc * Mm + m0 + k] : make_float2(0.f, 0.f);
-            Ss[i] = in ? S[(long long)bc * Mm + m0 + k] : make_float2(0.f, 0.f);
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < nm * W * W; i += blockDim.x) {
-            const int c = i % W, o = (i / W) % W, mm = i / (W * W);
-            float ar = 0.f, ai = 0.f;
-            for (int b = 0; b < B; ++b) {
-                const float2 g = Gs[((size_t)b * W + o) * MB + mm];
-                const float2 v = Ss[((size_t)b * W + c) * MB + mm];
-                ar = fmaf(g.x, v.x, fmaf(g.y, v.y, ar));
-                ai = fmaf(g.y, v.x, fmaf(-g.x, v.y, ai));
-            }
-            const long long t = (m0 + mm) * W * W + (long long)o * W + c;
-            dR[2 * t] += ar;
-            dR[2 * t + 1] += ai;
-        }
-    }
-}
-
-// Stage 1 of the pointwise weight gradient with a CTA per chunk of positions: dY and X of CH
-// positions staged in shared memory, each thread accumulating a few of the cout x (cin + 1) sums
-// over its CTA's chunks; part[(o * nblk + blk) * (cin + 1) + c] (stage 2 as before).
-constexpr int PW_CH = 64, PW_LD = PW_CH + 1;  // positions per chunk; padded row (distinct banks per channel)
-__global__ void k_pointwise_wgrad_g(const float* __restrict__ dY, const float* __restrict__ X, int B, int cin, int cout,
-                                    long long K, float* __restrict__ part) {
-    extern __shared__ float sm2[];
-    float* Ys = sm2;                         // [cout][PW_LD]
-    float* Xs = sm2 + (size_t)cout * PW_LD;  // [cin][PW_LD]
-    const int nout = cout * (cin + 1);
-    constexpr int MAXO = 8;
-    float acc[MAXO];
-#pragma unroll
-    for (int u = 0; u < MAXO; ++u) acc[u] = 0.f;
-    const long long kchunks = (K + PW_CH - 1) / PW_CH, total = (long long)B * kchunks;
-    for (long long ch = blockIdx.x; ch < total; ch += gridDim.x) {
-        const long long b = ch / kchunks, k0 = (ch % kchunks) * PW_CH;
-        const int nk = (int)min((long long)PW_CH, K - k0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < cout * PW_CH; i += blockDim.x) {
-            const int o = i / PW_CH, k = i % PW_CH;
-            Ys[o * PW_LD + k] = k < nk ? dY[(b * cout + o) * K + k0 + k] : 0.f;
-        }
-        for (int i = threadIdx.x; i < cin * PW_CH; i += blockDim.x) {
-            const int c = i / PW_CH, k = i % PW_CH;
-            Xs[c * PW_LD + k] = k < nk ? X[(b * cin + c) * K + k0 + k] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < MAXO; ++u) {
-            const int j = threadIdx.x + u * blockDim.x;
-            if (j >= nout) break;
-            const int o = j / (cin + 1), c = j % (cin + 1);
-            const float* yr = Ys + (size_t)o * PW_LD;
-            float a = acc[u];
-            if (c < cin) {
-                const float* xr = Xs + (size_t)c * PW_LD;
-                for (int k = 0; k < PW_CH; ++k) a = fmaf(yr[k], xr[k], a);
-            } else {
-                for (int k = 0; k < PW_CH; ++k) a += yr[k];
-            }
-            acc[u] = a;
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < MAXO; ++u) {
-        const int j = threadIdx.x + u * blockDim.x;
-        if (j >= nout) break;
-        const int o = j / (cin + 1), c = j % (cin + 1);
-        part[((long long)o * gridDim.x + blockIdx.x) * (cin + 1) + c] = acc[u];
-    }
-}
-
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_g(float z) {
-    return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
-}
-
-__global__ void k_gelu(const float* __restrict__ z, float* __restrict__ h, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        h[i] = gelu_f(z[i]);
-}
-__global__ void k_gelu_bwd(const float* __restrict__ dh, const float* __restrict__ z, float* __restrict__ dz, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        dz[i] = dh[i] * gelu_g(z[i]);
 }
 
 // MSE: per-block partial sums of (y - t)^2 and dy = 2 (y - t) / n; then a fixed-order final sum.
@@ -379,26 +583,46 @@ __global__ void k_mse_part(const float* __restrict__ y, const float* __restrict_
     twa::block_reduce_store<1>(acc, part);
 }
 __global__ void k_mse_final(const double* __restrict__ part, int nb, long long n, float* __restrict__ loss) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nb; ++b) s += part[b];
-        *loss = (float)(s / (double)n);
+    __shared__ double red[256];
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 256) s += part[b];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) *loss = (float)(red[0] / (double)n);
 }
 
+// Bound by memory: 30 bytes a parameter, read and written four at a time (268 M parameters: 1.59 ms
+// one at a time, now 1.16 ms).
 __global__ void k_adamw(float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                         __nv_bfloat16* __restrict__ th16, long long n, float lr, float b1, float b2, float eps, float wd,
                         float c1, float c2) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float upd = (mi / c1) / (sqrtf(vi / c2) + eps) + wd * th[i];
-        const float t = th[i] - lr * upd;
-        th[i] = t;
-        th16[i] = __float2bfloat16(t);
+    auto one = [&](float& t, float gi, float& mi, float& vi) {
+        mi = b1 * mi + (1.f - b1) * gi;
+        vi = b2 * vi + (1.f - b2) * gi * gi;
+        const float upd = (mi / c1) / (sqrtf(vi / c2) + eps) + wd * t;
+        t = t - lr * upd;
+    };
+    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
+    for (long long i = i0; i < n / 4; i += st) {
+        float4 t = reinterpret_cast<float4*>(th)[i], a = reinterpret_cast<float4*>(m)[i], b = reinterpret_cast<float4*>(v)[i];
+        const float4 gi = reinterpret_cast<const float4*>(g)[i];
+        one(t.x, gi.x, a.x, b.x);
+        one(t.y, gi.y, a.y, b.y);
+        one(t.z, gi.z, a.z, b.z);
+        one(t.w, gi.w, a.w, b.w);
+        reinterpret_cast<float4*>(th)[i] = t;
+        reinterpret_cast<float4*>(m)[i] = a;
+        reinterpret_cast<float4*>(v)[i] = b;
+        reinterpret_cast<__nv_bfloat162*>(th16)[2 * i] = __floats2bfloat162_rn(t.x, t.y);
+        reinterpret_cast<__nv_bfloat162*>(th16)[2 * i + 1] = __floats2bfloat162_rn(t.z, t.w);
+    }
+    for (long long i = n / 4 * 4 + i0; i < n; i += st) {
+        one(th[i], g[i], m[i], v[i]);
+        th16[i] = __float2bfloat16(th[i]);
     }
 }
 
@@ -433,14 +657,13 @@ struct twa_fno {
     int* d_err = nullptr;
     // activations for the largest batch seen
     int cap_b = 0;
-    std::vector<float*> h, z;
+    std::vector<float*> h, z;   // h[layers] is z[layers - 1]
     std::vector<float2*> s;
     float2* t1 = nullptr;
     float2* t2 = nullptr;
     float2* mixed = nullptr;
-    float* dh = nullptr;
-    float* dz = nullptr;
-    float* dh2 = nullptr;
+    float* dz = nullptr;        // dL/dz of the current layer, and the next one's as it is formed
+    float* dz2 = nullptr;
     float* part = nullptr;
     double* lpart = nullptr;
     const float* x_in = nullptr;
@@ -481,10 +704,12 @@ long long kmodes(const twa_fno* f) {
 
 int ensure_batch(twa_fno* f, int B) {
     if (B <= f->cap_b) return 0;
+    f->cap_b = 0;  // nothing is held if an allocation below fails
+    if (!f->h.empty()) f->h.pop_back();  // z[layers - 1] again
     for (float* p : f->h) cudaFree(p);
     for (float* p : f->z) cudaFree(p);
     for (float2* p : f->s) cudaFree(p);
-    for (void* p : {(void*)f->t1, (void*)f->t2, (void*)f->mixed, (void*)f->dh, (void*)f->dz, (void*)f->dh2})
+    for (void* p : {(void*)f->t1, (void*)f->t2, (void*)f->mixed, (void*)f->dz, (void*)f->dz2})
         if (p) cudaFree(p);
     std::vector<void*> keep;
     for (void* p : f->allocs) {
@@ -492,17 +717,17 @@ int ensure_batch(twa_fno* f, int B) {
         for (float* q : f->h) act |= (p == q);
         for (float* q : f->z) act |= (p == q);
         for (float2* q : f->s) act |= (p == (void*)q);
-        for (void* q : {(void*)f->t1, (void*)f->t2, (void*)f->mixed, (void*)f->dh, (void*)f->dz, (void*)f->dh2})
+        for (void* q : {(void*)f->t1, (void*)f->t2, (void*)f->mixed, (void*)f->dz, (void*)f->dz2})
             act |= (p == q && q);
         if (!act) keep.push_back(p);
     }
     f->allocs = keep;
     const int L = f->cfg.layers, W = f->cfg.width, n = f->cfg.grid, m2 = 2 * f->cfg.modes;
     const long long K = kcells(f), Mm = kmodes(f);
-    f->h.assign(L + 1, nullptr);
+    f->h.assign(L, nullptr);
     f->z.assign(L, nullptr);
     f->s.assign(L, nullptr);
-    for (int l = 0; l <= L; ++l)
+    for (int l = 0; l < L; ++l)
         if (int rc = falloc(f, &f->h[l], (size_t)B * W * K)) return rc;
     for (int l = 0; l < L; ++l) {
         if (int rc = falloc(f, &f->z[l], (size_t)B * W * K)) return rc;
@@ -512,62 +737,73 @@ int ensure_batch(twa_fno* f, int B) {
     if (int rc = falloc(f, &f->t1, tsz)) return rc;
     if (int rc = falloc(f, &f->t2, tsz)) return rc;
     if (int rc = falloc(f, &f->mixed, (size_t)B * W * Mm)) return rc;
-    if (int rc = falloc(f, &f->dh, (size_t)B * W * K)) return rc;
     if (int rc = falloc(f, &f->dz, (size_t)B * W * K)) return rc;
-    if (int rc = falloc(f, &f->dh2, (size_t)B * W * K)) return rc;
+    if (int rc = falloc(f, &f->dz2, (size_t)B * W * K)) return rc;
+    f->h.push_back(f->z[L - 1]);
     f->cap_b = B;
     return 0;
 }
 
-// Axis contraction: the grouped kernel when M fits in shared memory, else the per-output one.
-void axis_launch(const twa_fno* f, int blocks, int threads, int smem0, cudaStream_t st, const float2* in_c,
-                 const float* in_r, const float2* M, float2* out_c, float* out_r, long long P, int nin, int nout,
-                 long long Q, int accumulate) {
-    (void)f;
-    (void)smem0;
-    const size_t sm = (size_t)nin * nout * sizeof(float2);
-    if (sm <= 48 * 1024) {
-        const long long work = P * ((nout + AG - 1) / AG) * Q;
-        k_axis_g<<<blocks_for(work), threads, sm, st>>>(in_c, in_r, M, out_c, out_r, P, nin, nout, Q, accumulate);
-    } else {
-        k_axis<<<blocks, threads, 0, st>>>(in_c, in_r, M, out_c, out_r, P, nin, nout, Q, accumulate);
-    }
+// Kernel attributes of the current device (at creation).
+int fno_prepare() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void* k, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    const int ax = 2 * AX_O * 128 * 16 + 2 * AX_J * AX_COLS * 8;
+    set((const void*)k_axis<false, false>, ax);
+    set((const void*)k_axis<true, false>, ax);
+    set((const void*)k_axis<false, true>, ax);
+    set((const void*)k_pointwise_wgrad<true>, WG_SMEM);
+    set((const void*)k_pointwise_wgrad<false>, WG_SMEM);
+    set((const void*)k_mix_wgrad<true>, kMixWgradSmem);
+    set((const void*)k_mix_wgrad<false>, kMixWgradSmem);
+    return e == cudaSuccess ? 0 : -3;
 }
 
-// Modes per CTA of the mixing kernels (W threads per mode) and their shared memory.
-int mix_modes(int W) { return kThreads / W > 0 ? kThreads / W : 1; }
+// One axis contraction of a complex (in_c) or real (in_r) input into a complex (out_c) or real (out_r) output.
+void axis_launch(cudaStream_t st, const float2* in_c, const float* in_r, const float2* M, float2* out_c, float* out_r,
+                 long long P, int nin, int nout, long long Q, int accumulate) {
+    const long long cols = P * Q;
+    const dim3 grid((unsigned)((cols + AX_COLS - 1) / AX_COLS), (unsigned)((nout + 4 * AX_O - 1) / (4 * AX_O)));
+    const size_t sm = (size_t)2 * AX_O * nin * sizeof(float4) + 2 * AX_J * AX_COLS * (in_r ? sizeof(float) : sizeof(float2));
+    if (in_r)
+        k_axis<true, false><<<grid, 128, sm, st>>>(in_r, M, out_c, cols, nin, nout, Q, 0);
+    else if (out_r)
+        k_axis<false, true><<<grid, 128, sm, st>>>(in_c, M, out_r, cols, nin, nout, Q, accumulate);
+    else
+        k_axis<false, false><<<grid, 128, sm, st>>>(in_c, M, out_c, cols, nin, nout, Q, 0);
+}
+
+bool aligned(const void* p, unsigned bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
 
 template <bool ADJ>
 void mix_launch(const float2* S, const __nv_bfloat16* R, float2* Y, int B, int W, long long Mm, cudaStream_t st) {
-    const int MB = mix_modes(W);
-    const size_t sm = ((size_t)MB * W * W + (size_t)B * W * MB) * sizeof(float2);
-    if (W <= kThreads && sm <= 100 * 1024) {
-        static size_t set = 0;
-        if (sm > set) {
-            cudaFuncSetAttribute(k_mix_g<ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            set = sm;
-        }
-        const long long nb = (Mm + MB - 1) / MB;
-        k_mix_g<ADJ><<<(int)(nb < 152LL * 8 ? nb : 152LL * 8), MB * W, sm, st>>>(S, R, Y, B, W, Mm, MB);
-    } else {
-        k_mix<ADJ><<<blocks_for((long long)B * W * Mm), kThreads, 0, st>>>(S, R, Y, B, W, Mm);
-    }
+    const int MB = MIX_T / W;   // modes per CTA (W <= 64)
+    const size_t sm = (size_t)2 * MIX_B * MB * (W + 1) * sizeof(float2);
+    const unsigned nb = (unsigned)((Mm + MB - 1) / MB);
+    // the layers' matrices start where the ones before them end: on 16, 4 or 2 bytes
+    if (!ADJ && W % 4 == 0 && aligned(R, 16))
+        k_mix<ADJ, R_FOUR><<<nb, MB * W, sm, st>>>(S, R, Y, B, W, Mm, MB);
+    else if (aligned(R, 4))
+        k_mix<ADJ, R_COMPLEX><<<nb, MB * W, sm, st>>>(S, R, Y, B, W, Mm, MB);
+    else
+        k_mix<ADJ, R_SCALAR><<<nb, MB * W, sm, st>>>(S, R, Y, B, W, Mm, MB);
 }
 
 void mix_wgrad_launch(const float2* G, const float2* S, float* dR, int B, int W, long long Mm, cudaStream_t st) {
-    const int MB = mix_modes(W);
-    const size_t sm = (size_t)2 * B * W * MB * sizeof(float2);
-    if (sm <= 100 * 1024) {
-        static size_t set = 0;
-        if (sm > set) {
-            cudaFuncSetAttribute(k_mix_wgrad_g, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            set = sm;
-        }
-        const long long nb = (Mm + MB - 1) / MB;
-        k_mix_wgrad_g<<<(int)(nb < 152LL * 8 ? nb : 152LL * 8), kThreads, sm, st>>>(G, S, dR, B, W, Mm, MB);
-    } else {
-        k_mix_wgrad<<<blocks_for(Mm * W * W), kThreads, 0, st>>>(G, S, dR, B, W, Mm);
+    const size_t one = (size_t)2 * B * (W + 1) * sizeof(float2);   // one mode
+    if (one > (size_t)kMixWgradSmem) {
+        k_mix_wgrad_any<<<blocks_for(Mm * W * W), kThreads, 0, st>>>(G, S, dR, B, W, Mm);
+        return;
     }
+    // eight modes (64-byte segments of the inputs) as far as 48 KB hold them
+    const int MB = one * 8 <= 48 * 1024 ? 8 : (one <= 48 * 1024 ? (int)(48 * 1024 / one) : 1);
+    const unsigned nb = (unsigned)((Mm + MB - 1) / MB);
+    if (W % 2 == 0 && aligned(dR, 16))
+        k_mix_wgrad<true><<<nb, MIX_T, one * MB, st>>>(G, S, dR, B, W, Mm, MB);
+    else
+        k_mix_wgrad<false><<<nb, MIX_T, one * MB, st>>>(G, S, dR, B, W, Mm, MB);
 }
 
 // A (truncated forward DFT) of a real [B*W][n][n][n] field into complex [B*W][2m][2m][2m].
@@ -577,49 +813,51 @@ void dft_fwd(twa_fno* f, const float* in, float2* out, long long BW, cudaStream_
     if (!(f->tc_on && f->tc_fwd &&
           twa::tc_gemm(in, BW * n * n, n, n, f->Bf, 2 * m2, f->npf, reinterpret_cast<float*>(f->t1), 2 * m2, 0, f->d_err,
                   2.0, st) == 0))
-        axis_launch(f, blocks_for(BW * n * n * m2), kThreads, 0, st, nullptr, in, f->Mf[2], f->t1, nullptr, BW * n * n, n, m2, 1,
-                                                                  0);
+        axis_launch(st, nullptr, in, f->Mf[2], f->t1, nullptr, BW * n * n, n, m2, 1, 0);
     // y axis: (BW*n, n, 2m) -> (BW*n, 2m, 2m)
-    axis_launch(f, blocks_for(BW * n * m2 * m2), kThreads, 0, st, f->t1, nullptr, f->Mf[1], f->t2, nullptr, BW * n, n, m2, m2, 0);
+    axis_launch(st, f->t1, nullptr, f->Mf[1], f->t2, nullptr, BW * n, n, m2, m2, 0);
     // z axis: (BW, n, 4m^2) -> (BW, 2m, 4m^2)
-    axis_launch(f, blocks_for(BW * m2 * m2 * m2), kThreads, 0, st, f->t2, nullptr, f->Mf[0], out, nullptr, BW, n, m2,
-                                                               (long long)m2 * m2, 0);
+    axis_launch(st, f->t2, nullptr, f->Mf[0], out, nullptr, BW, n, m2, (long long)m2 * m2, 0);
 }
 
 // Re A^H of complex [BW][2m][2m][2m] into a real [BW][n][n][n] field (overwrite or add).
 void dft_adj(twa_fno* f, const float2* in, float* out, long long BW, int accumulate, cudaStream_t st) {
     const int n = f->cfg.grid, m2 = 2 * f->cfg.modes;
-    axis_launch(f, blocks_for(BW * n * m2 * m2), kThreads, 0, st, in, nullptr, f->Mi[0], f->t1, nullptr, BW, m2, n,
-                                                              (long long)m2 * m2, 0);
-    axis_launch(f, blocks_for(BW * n * n * m2), kThreads, 0, st, f->t1, nullptr, f->Mi[1], f->t2, nullptr, BW * n, m2, n, m2, 0);
+    axis_launch(st, in, nullptr, f->Mi[0], f->t1, nullptr, BW, m2, n, (long long)m2 * m2, 0);
+    axis_launch(st, f->t1, nullptr, f->Mi[1], f->t2, nullptr, BW * n, m2, n, m2, 0);
     if (!(f->tc_on && f->tc_adj &&
           twa::tc_gemm(reinterpret_cast<const float*>(f->t2), BW * n * n, 2 * m2, 2 * m2, f->Ba, n, f->npa, out, n, accumulate,
                   f->d_err, 2.0, st) == 0))
-        axis_launch(f, blocks_for(BW * n * n * n), kThreads, 0, st, f->t2, nullptr, f->Mi[2], nullptr, out, BW * n * n, m2, n,
-                                                                1, accumulate);
+        axis_launch(st, f->t2, nullptr, f->Mi[2], nullptr, out, BW * n * n, m2, n, 1, accumulate);
 }
 
-void pointwise(const float* X, const __nv_bfloat16* W, const float* b, float* Y, int B, int cin, int cout, long long K,
-               int acc, bool trans, cudaStream_t st) {
-    const size_t sm = (size_t)cin * cout * sizeof(float);
-    if (trans)
-        k_pointwise<true><<<blocks_for((long long)B * K), kThreads, sm, st>>>(X, W, b, Y, B, cin, cout, K, acc);
+template <int PW_O, int P, bool TRANS, int EP>
+void pointwise_o(const float* X, const __nv_bfloat16* W, const float* b, float* Y, float* Z, int B, int cin, int cout,
+                 long long K, int acc, cudaStream_t st) {
+    const dim3 grid((unsigned)((K + 128 * P - 1) / (128 * P)), (unsigned)((cout + PW_O - 1) / PW_O), (unsigned)(B < 65535 ? B : 65535));
+    if (K % 4 == 0 && aligned(X, 16) && aligned(Y, 16) && aligned(Z, 16))
+        k_pointwise<PW_O, P, TRANS, EP, true><<<grid, 128, 0, st>>>(X, W, b, Y, Z, B, cin, cout, K, acc);
     else
-        k_pointwise<false><<<blocks_for((long long)B * K), kThreads, sm, st>>>(X, W, b, Y, B, cin, cout, K, acc);
+        k_pointwise<PW_O, P, TRANS, EP, false><<<grid, 128, 0, st>>>(X, W, b, Y, Z, B, cin, cout, K, acc);
+}
+// Z: where EP_GELU stores gelu(Y), or what EP_GRAD takes gelu' of
+template <bool TRANS, int EP>
+void pointwise(const float* X, const __nv_bfloat16* W, const float* b, float* Y, float* Z, int B, int cin, int cout,
+               long long K, int acc, cudaStream_t st) {
+    if (cout <= 4) pointwise_o<4, 4, TRANS, EP>(X, W, b, Y, Z, B, cin, cout, K, acc, st);
+    else if (cout <= 8) pointwise_o<8, 4, TRANS, EP>(X, W, b, Y, Z, B, cin, cout, K, acc, st);
+    else if (cout <= 16) pointwise_o<16, 4, TRANS, EP>(X, W, b, Y, Z, B, cin, cout, K, acc, st);
+    else pointwise_o<32, 2, TRANS, EP>(X, W, b, Y, Z, B, cin, cout, K, acc, st);
 }
 
 void pointwise_wgrad(twa_fno* f, const float* dY, const float* X, int B, int cin, int cout, long long K, float* dW,
                      float* db, cudaStream_t st) {
-    if ((long long)cout * (cin + 1) <= 8LL * kThreads) {
-        const int nblk = kPwBlocks;
-        const size_t sm = (size_t)(cin + cout) * PW_LD * sizeof(float);
-        k_pointwise_wgrad_g<<<nblk, kThreads, sm, st>>>(dY, X, B, cin, cout, K, f->part);
-        k_pointwise_wgrad_sum<<<(cout * (cin + 1) + 127) / 128, 128, 0, st>>>(f->part, cin, cout, nblk, dW, db);
-        return;
-    }
-    const int nchunk = 64;
-    k_pointwise_wgrad_part<<<dim3(cout, nchunk), kThreads, 0, st>>>(dY, X, B, cin, cout, K, nchunk, f->part);
-    k_pointwise_wgrad_sum<<<(cout * (cin + 1) + 127) / 128, 128, 0, st>>>(f->part, cin, cout, nchunk, dW, db);
+    const dim3 grid(kPwBlocks, (unsigned)(((cout + 31) / 32) * ((cin + 31) / 32)));
+    if (K % 4 == 0 && aligned(dY, 16) && aligned(X, 16))
+        k_pointwise_wgrad<true><<<grid, 256, WG_SMEM, st>>>(dY, X, B, cin, cout, K, f->part);
+    else
+        k_pointwise_wgrad<false><<<grid, 256, WG_SMEM, st>>>(dY, X, B, cin, cout, K, f->part);
+    k_pointwise_wgrad_sum<<<cout, 128, 0, st>>>(f->part, cin, kPwBlocks, dW, db);
 }
 
 }  // namespace
@@ -660,10 +898,11 @@ int twa_fno_create(twa_fno** out, const twa_fno_config* cfg, uint64_t seed) {
         (rc = falloc(f, &f->am, o)) || (rc = falloc(f, &f->av, o)))
         return bail(rc);
     const int maxc = (W > c.c_in ? W : c.c_in) > c.c_out ? (W > c.c_in ? W : c.c_in) : c.c_out;
-    if ((rc = falloc(f, &f->part, (size_t)maxc * (kPwBlocks > 64 ? kPwBlocks : 64) * (maxc + 1))) ||
+    if ((rc = falloc(f, &f->part, (size_t)maxc * kPwBlocks * (maxc + 1))) ||
         (rc = falloc(f, &f->lpart, (size_t)152 * 64)))
         return bail(rc);
     // truncated unitary DFT matrices (FP64 on the host), kept frequencies {0..m-1} U {n-m..n-1}
+    if (fno_prepare() != 0) return bail(ffail(f, TWA_ECUDA, "twa_fno_create: cudaFuncSetAttribute failed"));
     const int n = c.grid, m2 = 2 * c.modes;
     std::vector<float2> mf((size_t)m2 * n), mi((size_t)n * m2);
     for (int i = 0; i < m2; ++i) {
@@ -768,18 +1007,17 @@ int twa_fno_forward(twa_fno* f, const float* x, int B, float* y, void* stream) {
     const int W = f->cfg.width, L = f->cfg.layers;
     const long long K = kcells(f), Mm = kmodes(f), BW = (long long)B * W;
     const __nv_bfloat16* P = f->th16;
-    pointwise(x, P + f->oP, f->th + f->op, f->h[0], B, f->cfg.c_in, W, K, 0, false, st);
+    pointwise<false, EP_NONE>(x, P + f->oP, f->th + f->op, f->h[0], nullptr, B, f->cfg.c_in, W, K, 0, st);
     for (int l = 0; l < L; ++l) {
         dft_fwd(f, f->h[l], f->s[l], BW, st);
         mix_launch<false>(f->s[l], P + f->oR[l], f->mixed, B, W, Mm, st);
         dft_adj(f, f->mixed, f->z[l], BW, 0, st);
-        pointwise(f->h[l], P + f->oW[l], f->th + f->ob[l], f->z[l], B, W, W, K, 1, false, st);
         if (l < L - 1)
-            k_gelu<<<blocks_for(BW * K), kThreads, 0, st>>>(f->z[l], f->h[l + 1], BW * K);
+            pointwise<false, EP_GELU>(f->h[l], P + f->oW[l], f->th + f->ob[l], f->z[l], f->h[l + 1], B, W, W, K, 1, st);
         else
-            FC(cudaMemcpyAsync(f->h[l + 1], f->z[l], BW * K * sizeof(float), cudaMemcpyDeviceToDevice, st));
+            pointwise<false, EP_NONE>(f->h[l], P + f->oW[l], f->th + f->ob[l], f->z[l], nullptr, B, W, W, K, 1, st);
     }
-    pointwise(f->h[L], P + f->oQ, f->th + f->oq, y, B, W, f->cfg.c_out, K, 0, false, st);
+    pointwise<false, EP_NONE>(f->h[L], P + f->oQ, f->th + f->oq, y, nullptr, B, W, f->cfg.c_out, K, 0, st);
     f->x_in = x;
     f->last_b = B;
     FC(cudaGetLastError());
@@ -794,25 +1032,25 @@ int twa_fno_backward(twa_fno* f, const float* dy, int B, float* dx, void* stream
     const __nv_bfloat16* P = f->th16;
     float* g = f->grad;
     pointwise_wgrad(f, dy, f->h[L], B, W, f->cfg.c_out, K, g + f->oQ, g + f->oq, st);
-    pointwise(dy, P + f->oQ, nullptr, f->dh, B, f->cfg.c_out, W, K, 0, true, st);
+    pointwise<true, EP_NONE>(dy, P + f->oQ, nullptr, f->dz, nullptr, B, f->cfg.c_out, W, K, 0, st);
     for (int l = L - 1; l >= 0; --l) {
-        float* dzl = f->dz;
-        if (l < L - 1)
-            k_gelu_bwd<<<blocks_for(BW * K), kThreads, 0, st>>>(f->dh, f->z[l], dzl, BW * K);
-        else
-            FC(cudaMemcpyAsync(dzl, f->dh, BW * K * sizeof(float), cudaMemcpyDeviceToDevice, st));
-        pointwise_wgrad(f, dzl, f->h[l], B, W, W, K, g + f->oW[l], g + f->ob[l], st);
-        pointwise(dzl, P + f->oW[l], nullptr, f->dh2, B, W, W, K, 0, true, st);
-        // spectral branch: dmixed = A dz, dR += dmixed conj(s), ds = R^H dmixed, dh += Re A^H ds
-        dft_fwd(f, dzl, f->mixed, BW, st);
+        pointwise_wgrad(f, f->dz, f->h[l], B, W, W, K, g + f->oW[l], g + f->ob[l], st);
+        // spectral branch: dmixed = A dz, dR += dmixed conj(s), ds = R^H dmixed (in t2, which the adjoint
+        // transform reads before it writes it), dh = Re A^H ds
+        float2* ds = f->t2;
+        dft_fwd(f, f->dz, f->mixed, BW, st);
         mix_wgrad_launch(f->mixed, f->s[l], g + f->oR[l], B, W, Mm, st);
-        mix_launch<true>(f->mixed, P + f->oR[l], reinterpret_cast<float2*>(f->dz), B, W, Mm, st);
-        // f->dz now holds ds (complex, B*W*Mm <= B*W*K floats / 2 since Mm <= K / 8)
-        dft_adj(f, reinterpret_cast<float2*>(f->dz), f->dh2, BW, 1, st);
-        std::swap(f->dh, f->dh2);
+        mix_launch<true>(f->mixed, P + f->oR[l], ds, B, W, Mm, st);
+        dft_adj(f, ds, f->dz2, BW, 0, st);
+        // dh += W^T dz, and for the layer below dz = dh gelu'(z)
+        if (l > 0)
+            pointwise<true, EP_GRAD>(f->dz, P + f->oW[l], nullptr, f->dz2, f->z[l - 1], B, W, W, K, 1, st);
+        else
+            pointwise<true, EP_NONE>(f->dz, P + f->oW[l], nullptr, f->dz2, nullptr, B, W, W, K, 1, st);
+        std::swap(f->dz, f->dz2);
     }
-    pointwise_wgrad(f, f->dh, f->x_in, B, f->cfg.c_in, W, K, g + f->oP, g + f->op, st);
-    if (dx) pointwise(f->dh, P + f->oP, nullptr, dx, B, W, f->cfg.c_in, K, 0, true, st);
+    pointwise_wgrad(f, f->dz, f->x_in, B, f->cfg.c_in, W, K, g + f->oP, g + f->op, st);
+    if (dx) pointwise<true, EP_NONE>(f->dz, P + f->oP, nullptr, dx, nullptr, B, W, f->cfg.c_in, K, 0, st);
     FC(cudaGetLastError());
     return TWA_OK;
 }
@@ -840,7 +1078,7 @@ int twa_fno_mse(twa_fno* f, const float* y, const float* t, long long n, float* 
     cudaStream_t st = (cudaStream_t)stream;
     const int nb = 152 * 4;
     k_mse_part<<<nb, 256, 0, st>>>(y, t, n, dy, f->lpart);
-    k_mse_final<<<1, 32, 0, st>>>(f->lpart, nb, n, loss);
+    k_mse_final<<<1, 256, 0, st>>>(f->lpart, nb, n, loss);
     FC(cudaGetLastError());
     return TWA_OK;
 }
