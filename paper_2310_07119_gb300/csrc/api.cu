@@ -223,13 +223,6 @@ struct twa_handle;
 namespace {
 void split_kick(const twa_handle* h, const Inst& I, double frac, float& hi, float& lo);
 
-int default_lines(int N, bool strided, int op) {
-    const int T = plan_threads_per_line(N);
-    if (op == OP_STEPS_1D) return std::max(1, 128 / T);
-    if (strided) return std::max(4, 256 / T);
-    return std::max(1, 256 / T);
-}
-
 int dispatch(int N, const LaunchCfg& c, const PassArgs& a, cudaStream_t st, bool prep) {
     switch (N) {
         case 8: return launch_line<8>(c, a, st, prep);
@@ -329,6 +322,52 @@ bool variant_ok(int N, int op, bool strided, int lines) {
     }
 }
 
+// Shape and variant of a pass when the tuner has not chosen one.  CTAs of 128 threads win almost
+// everywhere (256 threads leave two per SM, so that the barriers of one are covered by one other;
+// 64 or 32 make the segments of a column or the shared tables too small).  us a launch, 128^3 x 257
+// slots unless stated, half the threads against 256:
+//   drift_rho z 2394 -> 2080, drift y 2017 -> 1733, fwd y 1615 -> 1427, inv 833 -> 742, kick_drift x 1741 -> 1704;
+//   64^3 x 257: drift 288 -> 245, fwd_mul_inv 141 -> 129; 256^3 x 65: drift_rho 5258 -> 4915, inv 1826 -> 1624.
+// Exceptions, each measured the same way:
+//   rows of 1024 and 2048 cells: one line per CTA (kick_drift 1024^2 x 65: four lines 385, two 333, one 316;
+//     2048^2 x 17: two lines 420, one 372);
+//   columns of 512 cells: eight lines, 64-byte segments (drift_rho 512^2 x 129: four 263, eight 241);
+//   the two-field drift (both slots of a pair share the table reads): N = 32 15 -> 13, N = 64 245 -> 188,
+//     N = 128 1733 -> 1556, N = 256 (16 lines) 3991 -> 3765.  The missing partner of an odd slot count is
+//     transformed as zeros, so it needs an even count or enough slots (3 slots of 128^3: 25 -> 28); the
+//     same holds for drift_rho up to 64 (N = 64: 271 -> 264) and kick_drift_vinv at 64 (270 -> 245);
+//   columns of 1024 and 2048 cells: TMA tiles (2048^2 x 17: drift_rho 736 -> 672, fwd 387 -> 304, inv 215 -> 179;
+//     1024^2 x 65: 624 -> 573, 300 -> 242, 179 -> 157), and 64-cell fwd_mul_inv (129 -> 111);
+//   pipelined columns of the single transforms: inv 742 -> 691 at 128, 1624 -> 1505 at 256, fwd 3220 -> 2966 at 256.
+int default_lines(const Inst& I, int axis, int op) {
+    const int N = I.n[axis], T = plan_threads_per_line(N);
+    if (op == OP_STEPS_1D) return std::max(1, 128 / T);
+    const bool pairs = I.n_slots % 2 == 0 || I.n_slots >= 9;
+    if (axis == 0) {
+        if (N >= 1024) return 1;
+        if (op == OP_KICK_DRIFT_VINV && N == 64 && pairs) return DUAL_FLAG | 16;
+        return std::max(1, 128 / T);
+    }
+    int l = N == 512 ? 8 : std::max(4, 128 / T), flag = 0;
+    if (op == OP_DRIFT && N >= 32 && N <= 256 && pairs) {
+        if (N == 256) l = 16;
+        flag = DUAL_FLAG;
+    } else if (op == OP_DRIFT_RHO && (N == 32 || N == 64) && pairs) {
+        flag = DUAL_FLAG;
+    } else if (N >= 1024 && (op == OP_DRIFT_RHO || op == OP_FWD || op == OP_INV)) {
+        flag = PIPE_FLAG | TMA_FLAG;
+    } else if (N == 64 && op == OP_FWD_MUL_INV) {
+        flag = PIPE_FLAG | TMA_FLAG;
+    } else if ((op == OP_INV && (N == 128 || N == 256)) || (op == OP_FWD && N == 256)) {
+        flag = PIPE_FLAG;
+    }
+    // pipelined passes need whole tiles; TMA needs the driver's encoder
+    long long stride = 1;
+    for (int b = 0; b < axis; ++b) stride *= I.n[b];
+    if ((flag & PIPE_FLAG) && (stride % l != 0 || !variant_ok(N, op, true, flag | l))) flag = 0;
+    return flag | l;
+}
+
 #define RC(x)                \
     do {                     \
         int rc_ = (x);       \
@@ -414,7 +453,7 @@ int run_pass(twa_handle* h, Inst& I, float2* psi, int axis, int op, double kick_
     int lines = force_lines;
     if (!lines) {
         auto it = I.lines.find(key_of(axis, op));
-        lines = (it != I.lines.end()) ? it->second : default_lines(N, strided, op);
+        lines = (it != I.lines.end()) ? it->second : default_lines(I, axis, op);
     }
     const bool pipe = (lines & PIPE_FLAG) != 0;
     const bool dual = (lines & DUAL_FLAG) != 0;
@@ -530,7 +569,10 @@ int run_plane(twa_handle* h, Inst& I, float2* psi, int pop, double kick_frac, cu
     int lines = force_lines;
     if (!lines) {
         auto it = I.lines.find(key_of(3, pop));
-        lines = (it != I.lines.end()) ? it->second : std::min(N, std::max(1, 256 / plan_threads_per_line(N)));
+        // 128 threads per CTA once they fill the GPU (four per SM), else 256: 128^3 x 257 slots 3957 -> 3655 us
+        // and 1880 -> 1744 (Poisson), 256^3 x 65 7829 -> 7641 and 4475 -> 4215; 128^3 x 3 58 against 62
+        const int thr = (long long)I.n[2] * I.n_pairs >= 4 * 152 ? 128 : 256;
+        lines = (it != I.lines.end()) ? it->second : std::min(N, std::max(1, thr / plan_threads_per_line(N)));
     }
     if (!plane_variant_ok(N, pop, lines))
         return fail(h, TWA_EINVAL, "no plane variant for N=" + std::to_string(N) + " lines=" + std::to_string(lines));
@@ -1075,7 +1117,9 @@ int twa_create(twa_handle** out, const twa_grid* grids, const twa_params* p, int
         I.off = off;
         off += (size_t)I.n_slots * I.cells;
         I.mode = (g.dim == 1) ? MODE_1D : (g.dim == 2 ? MODE_2D : MODE_3D);
-        if (g.dim == 3 && I.n[0] == I.n[1] && I.n[0] >= 16 && I.n[0] <= 256) I.mode = MODE_3DP;
+        // square xy planes: plane passes; from 128 cells on the fields go by axis passes (the same bits;
+        // a step of 128^3 x 257 slots 8171 -> 8064 us, of 128^3 x 3 140 -> 135, of 256^3 x 3 1093 -> 1041)
+        if (g.dim == 3 && I.n[0] == I.n[1] && I.n[0] >= 16 && I.n[0] <= 256) I.mode = I.n[0] >= 128 ? MODE_3DH : MODE_3DP;
         h->in.push_back(I);
     }
     // fork batches whose instances are all small (at most 2^22 complex values each)
