@@ -158,52 +158,107 @@ struct DF {
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
-// FP64 counterpart of DF for the plain FP64 path.
-struct DAcc {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double a) { v += a; }
-    __device__ __forceinline__ double value() const { return v; }
-};
-template <class T2> struct AccOf;
-template <> struct AccOf<float2> { using type = DF; using real = float; };
-template <> struct AccOf<double2> { using type = DAcc; using real = double; };
-
 // Amplitude and phase moments (Eq. varA, Eq. varPhi) of a synchronized instance, one thread per
 // cell, two passes over the streams (slots 1..n): the first sums psi, |psi| and |psi|^2, the
 // second the squared deviations (A_s - <A>)^2 and dphi_s^2, dphi_s = arg(psi_s conj(<psi>)) (0
 // reference where the mean field vanishes).  Per block: sum of <rho> Var(A) / <A> and of
 // <rho> <dphi^2>, <rho> the Weyl-corrected mean density.
-template <class T2>
-__global__ void k_phase_moments(const T2* __restrict__ psi, long long cells, int n_slots, double weyl,
-                                double* var_a, double* phi2, double* part) {
-    using Acc = typename AccOf<T2>::type;
-    using R = typename AccOf<T2>::real;
+__global__ void k_phase_moments_f64(const double2* __restrict__ psi, long long cells, int n_slots, double weyl,
+                                    double* var_a, double* phi2, double* part) {
     const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     double v[2] = {0.0, 0.0};
     if (g < cells) {
         const int ns = n_slots - 1;
-        Acc sa, sa2, sx, sy;
+        double sa = 0.0, sa2 = 0.0, sx = 0.0, sy = 0.0;
         for (int s = 1; s < n_slots; ++s) {
-            const T2 z = psi[(long long)s * cells + g];
-            const R a2 = z.x * z.x + z.y * z.y;
-            sa.add(sqrt(a2));
-            sa2.add(a2);
-            sx.add(z.x);
-            sy.add(z.y);
+            const double2 z = psi[(long long)s * cells + g];
+            const double a2 = z.x * z.x + z.y * z.y;
+            sa += sqrt(a2);
+            sa2 += a2;
+            sx += z.x;
+            sy += z.y;
         }
-        const double am = sa.value() / ns, mx = sx.value() / ns, my = sy.value() / ns;
+        const double am = sa / ns, mx = sx / ns, my = sy / ns;
         const double mm = sqrt(mx * mx + my * my);
-        const R ux = (R)(mm > 0.0 ? mx / mm : 1.0), uy = (R)(mm > 0.0 ? my / mm : 0.0);
-        Acc da, dp;
+        const double ux = mm > 0.0 ? mx / mm : 1.0, uy = mm > 0.0 ? my / mm : 0.0;
+        double da = 0.0, dp = 0.0;
         for (int s = 1; s < n_slots; ++s) {
-            const T2 z = psi[(long long)s * cells + g];
-            const R d = sqrt(z.x * z.x + z.y * z.y) - (R)am;
-            da.add(d * d);
-            const R ph = atan2(z.y * ux - z.x * uy, z.x * ux + z.y * uy);  // arg(z conj(u))
-            dp.add(ph * ph);
+            const double2 z = psi[(long long)s * cells + g];
+            const double d = sqrt(z.x * z.x + z.y * z.y) - am;
+            da += d * d;
+            const double ph = atan2(z.y * ux - z.x * uy, z.x * ux + z.y * uy);  // arg(z conj(u))
+            dp += ph * ph;
         }
-        const double va = da.value() / ns, p2 = dp.value() / ns;
-        const double rho = sa2.value() / ns - weyl;
+        const double va = da / ns, p2 = dp / ns;
+        const double rho = sa2 / ns - weyl;
+        if (var_a) var_a[g] = va;
+        if (phi2) phi2[g] = p2;
+        v[0] = am > 0.0 ? rho * va / am : 0.0;
+        v[1] = rho * p2;
+    }
+    block_reduce_store<2>(v, part);
+}
+
+// Two float-pair sums at once (DF, in packed two-lane FP32: half the issue slots).  add_sq adds a * a,
+// its product unrounded (both uses inside an fma).
+struct DF2 {
+    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
+    __device__ __forceinline__ void finish(float2 s, float2 bp, float2 abp) {
+        const float2 e = f2_add(f2_add(f2_sub(hi, f2_sub(s, bp)), abp), lo);
+        hi = f2_add(s, e);
+        lo = f2_sub(e, f2_sub(hi, s));
+    }
+    __device__ __forceinline__ void add(float2 a) {
+        const float2 s = f2_add(hi, a), bp = f2_sub(s, hi);
+        finish(s, bp, f2_sub(a, bp));
+    }
+    __device__ __forceinline__ void add_sq(float2 a) {
+        const float2 s = f2_fma(a, a, hi), bp = f2_sub(s, hi);
+        finish(s, bp, f2_fma(a, a, make_float2(-bp.x, -bp.y)));
+    }
+    __device__ __forceinline__ double x() const { return (double)hi.x + (double)lo.x; }
+    __device__ __forceinline__ double y() const { return (double)hi.y + (double)lo.y; }
+};
+
+// The same for float fields.  Bound by instruction issue (a square root and an arctangent a value, two
+// pairs of sums in the first pass and one in the second), so the sums run two to an instruction and
+// PM_U streams are loaded at once to keep the issue slots fed (128^3 x 64: 860 us one at a time, 615 now;
+// two reads at the copy rate take 320).
+constexpr int PM_U = 8;
+__global__ void __launch_bounds__(256) k_phase_moments_f32(const float2* __restrict__ psi, long long cells, int n_slots,
+                                                           double weyl, double* var_a, double* phi2, double* part) {
+    const long long g = blockIdx.x * 256LL + threadIdx.x;
+    double v[2] = {0.0, 0.0};
+    if (g < cells) {
+        const int ns = n_slots - 1;
+        auto each = [&](auto f) {  // f of every stream, in slot order
+            const float2* p = psi + cells + g;
+            int s = 0;
+            for (; s + PM_U <= ns; s += PM_U, p += PM_U * cells) {
+                float2 z[PM_U];
+#pragma unroll
+                for (int u = 0; u < PM_U; ++u) z[u] = __ldcs(&p[u * cells]);
+#pragma unroll
+                for (int u = 0; u < PM_U; ++u) f(z[u]);
+            }
+            for (; s < ns; ++s, p += cells) f(__ldcs(p));
+        };
+        DF2 sa, sz;  // (|psi|, |psi|^2), psi
+        each([&](float2 z) {
+            const float a2 = z.x * z.x + z.y * z.y;
+            sa.add(make_float2(sqrtf(a2), a2));
+            sz.add(z);
+        });
+        const double am = sa.x() / ns, mx = sz.x() / ns, my = sz.y() / ns;
+        const double mm = sqrt(mx * mx + my * my);
+        const float ux = (float)(mm > 0.0 ? mx / mm : 1.0), uy = (float)(mm > 0.0 ? my / mm : 0.0), amf = (float)am;
+        DF2 sd;      // (|psi| - <|psi|>)^2, phase^2
+        each([&](float2 z) {
+            const float d = sqrtf(z.x * z.x + z.y * z.y) - amf;
+            sd.add_sq(make_float2(d, atan2f(z.y * ux - z.x * uy, z.x * ux + z.y * uy)));  // arg(z conj(u))
+        });
+        const double va = sd.x() / ns, p2 = sd.y() / ns;
+        const double rho = sa.y() / ns - weyl;
         if (var_a) var_a[g] = va;
         if (phi2) phi2[g] = p2;
         v[0] = am > 0.0 ? rho * va / am : 0.0;
@@ -579,21 +634,19 @@ int launch_moments_modes(const float2* spec, long long cells, int n_slots, doubl
                                                            nk_var, nk_cl, part);
     return 0;
 }
-template <class T2>
-int launch_phase_moments_t(const T2* psi, long long cells, int n_slots, double weyl, double dV, double* var_a,
-                           double* phi2, double* part, double* out, cudaStream_t st) {
+int launch_phase_moments(const float2* psi, long long cells, int n_slots, double weyl, double dV, double* var_a,
+                         double* phi2, double* part, double* out, cudaStream_t st) {
     const int nb = moments_blocks(cells);
-    k_phase_moments<T2><<<nb, 256, 0, st>>>(psi, cells, n_slots, weyl, var_a, phi2, part);
+    k_phase_moments_f32<<<nb, 256, 0, st>>>(psi, cells, n_slots, weyl, var_a, phi2, part);
     k_finish_phase<<<1, 256, 0, st>>>(part, nb, dV, out);
     return 0;
 }
-int launch_phase_moments(const float2* psi, long long cells, int n_slots, double weyl, double dV, double* var_a,
-                         double* phi2, double* part, double* out, cudaStream_t st) {
-    return launch_phase_moments_t(psi, cells, n_slots, weyl, dV, var_a, phi2, part, out, st);
-}
 int launch_phase_moments_f64(const double2* psi, long long cells, int n_slots, double weyl, double dV,
                              double* var_a, double* phi2, double* part, double* out, cudaStream_t st) {
-    return launch_phase_moments_t(psi, cells, n_slots, weyl, dV, var_a, phi2, part, out, st);
+    const int nb = moments_blocks(cells);
+    k_phase_moments_f64<<<nb, 256, 0, st>>>(psi, cells, n_slots, weyl, var_a, phi2, part);
+    k_finish_phase<<<1, 256, 0, st>>>(part, nb, dV, out);
+    return 0;
 }
 int launch_finish_scalars(const double* part_r, int nb_r, const double* part_m, int nb_m, double dV,
                           double q_offset, double* scalars, int* err_word, cudaStream_t st) {
