@@ -564,7 +564,8 @@ bool plane_variant_ok(int N, int pop, int lines) {
 }
 
 // One xy-plane pass over all z-planes of every pair of instance I (3D, nx = ny).
-int run_plane(twa_handle* h, Inst& I, float2* psi, int pop, double kick_frac, cudaStream_t st, int force_lines = 0) {
+int run_plane(twa_handle* h, Inst& I, float2* psi, int pop, double kick_frac, cudaStream_t st, int force_lines = 0,
+              float2* out = nullptr) {
     const int N = I.n[0];
     int lines = force_lines;
     if (!lines) {
@@ -579,6 +580,7 @@ int run_plane(twa_handle* h, Inst& I, float2* psi, int pop, double kick_frac, cu
     PassArgs a{};
     a.psi = psi;
     a.buf = I.vc;
+    a.out = out;
     a.tw = h->tw32[N];
     a.ph = I.ph[0];
     a.ph2 = I.ph[1];
@@ -610,6 +612,19 @@ int run_plane(twa_handle* h, Inst& I, float2* psi, int pop, double kick_frac, cu
     }
     ++h->launches;
     return 0;
+}
+
+int dispatch_line_modes(int N, const PassArgs& a, const ModesArgs& m, int tiles, cudaStream_t st) {
+    switch (N) {
+        case 8: return launch_line_modes<8>(a, m, tiles, st);
+        case 16: return launch_line_modes<16>(a, m, tiles, st);
+        case 32: return launch_line_modes<32>(a, m, tiles, st);
+        case 64: return launch_line_modes<64>(a, m, tiles, st);
+        case 128: return launch_line_modes<128>(a, m, tiles, st);
+        case 256: return launch_line_modes<256>(a, m, tiles, st);
+        case 512: return launch_line_modes<512>(a, m, tiles, st);
+        default: return -1;
+    }
 }
 
 float2* inst_psi(Inst& I, void* psi) { return static_cast<float2*>(psi) + I.off; }
@@ -861,6 +876,17 @@ int batch_steps(twa_handle* h, void* psi, int n, double a_first, cudaStream_t st
     return 0;
 }
 
+// CTAs of the fused last axis of the mode moments (k_line_modes), 0 where the separate passes stay: 1D; less
+// than about one wave of CTAs (each walks through all slots); lengths past 512, whose lines take 256 or 512
+// threads and leave one CTA per SM (1024^2 x 65: 386 us in two passes, more in one).
+int modes_tiles(const Inst& I) {
+    const int N = I.n[I.dim - 1];
+    if (I.dim < 2 || N > 512) return 0;
+    const int L = std::max(4, 128 / plan_threads_per_line(N));
+    const long long tiles = (I.cells / N + L - 1) / L;
+    return tiles >= 600 ? (int)tiles : 0;
+}
+
 // Moments with a pending kick (0 for a synchronized batch); scalars into `scalars` (device).
 int moments_f32(twa_handle* h, Inst& I, float2* psi, double pend, const twa_moments_out* o, double* scalars,
                 cudaStream_t st) {
@@ -876,12 +902,29 @@ int moments_f32(twa_handle* h, Inst& I, float2* psi, double pend, const twa_mome
     ++h->launches;
     int nbm = 0;
     if (h->p.want_modes && I.spec) {
-        RC(run_pass(h, I, psi, 0, OP_KICK_FWD_OUT, pend, I.vc, I.spec, I.n_pairs, st, 0, I.mode == MODE_1D ? 1 : 0));
-        for (int ax = 1; ax < I.dim; ++ax) RC(run_pass(h, I, psi, ax, OP_FWD, 0.0, I.spec, nullptr, I.n_slots, st));
-        launch_moments_modes(I.spec, I.cells, I.n_slots, h->p.n_tot * I.dV / (double)I.cells, 1.0 / ns,
-                             o ? o->nk_mean : nullptr, o ? o->nk_var : nullptr, o ? o->nk_cl : nullptr, I.part_m, st);
+        const double anorm2 = h->p.n_tot * I.dV / (double)I.cells;
+        double *nk = o ? o->nk_mean : nullptr, *nv = o ? o->nk_var : nullptr, *nc = o ? o->nk_cl : nullptr;
+        // the pass profiler takes the transforms one by one
+        const int tiles = h->prof_on ? 0 : modes_tiles(I);
+        int ax = 1;
+        if (!h->prof_on && I.dim == 3 && I.n[0] == I.n[1] && I.n[0] >= 16 && I.n[0] <= 256) {
+            RC(run_plane(h, I, psi, PL_KICK_FWD, pend, st, 0, I.spec));
+            ax = 2;
+        } else {
+            RC(run_pass(h, I, psi, 0, OP_KICK_FWD_OUT, pend, I.vc, I.spec, I.n_pairs, st, 0, I.mode == MODE_1D ? 1 : 0));
+        }
+        for (; ax < I.dim - (tiles ? 1 : 0); ++ax)
+            RC(run_pass(h, I, psi, ax, OP_FWD, 0.0, I.spec, nullptr, I.n_slots, st));
+        if (tiles) {
+            const PassArgs a = make_args(h, I, nullptr, ax, 0.0, I.spec, nullptr);
+            const ModesArgs m{anorm2, 1.0 / ns, nk, nv, nc, I.part_m};
+            if (dispatch_line_modes(I.n[ax], a, m, tiles, st) != 0) return fail(h, TWA_EINVAL, "mode moments: no variant");
+            nbm = tiles;
+        } else {
+            launch_moments_modes(I.spec, I.cells, I.n_slots, anorm2, 1.0 / ns, nk, nv, nc, I.part_m, st);
+            nbm = nb;
+        }
         ++h->launches;
-        nbm = nb;
     }
     launch_finish_scalars(I.part_r, nb, I.part_m, nbm, I.dV, (double)I.cells / (2.0 * h->p.n_tot), scalars, h->d_err, st);
     ++h->launches;

@@ -4,6 +4,7 @@
 
 #include "fft_engine.cuh"
 #include "kernels.h"
+#include "pairsum.cuh"
 #include "passes.cuh"
 #include "reduce.cuh"
 #include "wigner.cuh"
@@ -133,31 +134,6 @@ __global__ void __launch_bounds__(256) k_kick_pairs(float2* __restrict__ psi, co
     }
 }
 
-// Running sum of floats carried as an unevaluated pair hi + lo ("double-float"): each addition's
-// rounding error is recovered exactly (Knuth's two-sum) and the pair is renormalized (Dekker's
-// fast two-sum), so the sum keeps about 48 significant bits.  The moment kernels accumulate in
-// this form because this part's FP64 rate is 1/64 of its FP32 rate: FP64 adds would make them
-// compute-bound at several times their memory time.  Results are finished in FP64.
-struct DF {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float a) {
-        const float s = hi + a;
-        const float bp = s - hi;
-        float e = (hi - (s - bp)) + (a - bp);  // hi + a = s + e exactly
-        e += lo;
-        hi = s + e;
-        lo = e - (hi - s);
-    }
-    // add a * a exactly (the product's rounding error recovered with an fma)
-    __device__ __forceinline__ void add_sq(float a) {
-        const float p = a * a;
-        const float q = fmaf(a, a, -p);
-        add(p);
-        lo += q;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Amplitude and phase moments (Eq. varA, Eq. varPhi) of a synchronized instance, one thread per
 // cell, two passes over the streams (slots 1..n): the first sums psi, |psi| and |psi|^2, the
 // second the squared deviations (A_s - <A>)^2 and dphi_s^2, dphi_s = arg(psi_s conj(<psi>)) (0
@@ -198,27 +174,6 @@ __global__ void k_phase_moments_f64(const double2* __restrict__ psi, long long c
     }
     block_reduce_store<2>(v, part);
 }
-
-// Two float-pair sums at once (DF, in packed two-lane FP32: half the issue slots).  add_sq adds a * a,
-// its product unrounded (both uses inside an fma).
-struct DF2 {
-    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
-    __device__ __forceinline__ void finish(float2 s, float2 bp, float2 abp) {
-        const float2 e = f2_add(f2_add(f2_sub(hi, f2_sub(s, bp)), abp), lo);
-        hi = f2_add(s, e);
-        lo = f2_sub(e, f2_sub(hi, s));
-    }
-    __device__ __forceinline__ void add(float2 a) {
-        const float2 s = f2_add(hi, a), bp = f2_sub(s, hi);
-        finish(s, bp, f2_sub(a, bp));
-    }
-    __device__ __forceinline__ void add_sq(float2 a) {
-        const float2 s = f2_fma(a, a, hi), bp = f2_sub(s, hi);
-        finish(s, bp, f2_fma(a, a, make_float2(-bp.x, -bp.y)));
-    }
-    __device__ __forceinline__ double x() const { return (double)hi.x + (double)lo.x; }
-    __device__ __forceinline__ double y() const { return (double)hi.y + (double)lo.y; }
-};
 
 // The same for float fields.  Bound by instruction issue (a square root and an arctangent a value, two
 // pairs of sums in the first pass and one in the second), so the sums run two to an instruction and
@@ -301,13 +256,13 @@ __global__ void k_moments_real(const float2* __restrict__ psi, const float2* __r
     const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     double v[NP_REAL] = {0, 0, 0, 0, 0, 0};
     if (g < cells) {
-        DF m2, pr, pi;
+        DF m2;
+        DF2 pz;
         int bad = 0;
         auto add = [&](float2 z, float2 zk) {
             bad += (!isfinite(z.x) || !isfinite(z.y)) ? 1 : 0;
             m2.add(fmaf(z.x, z.x, z.y * z.y));
-            pr.add(zk.x);
-            pi.add(zk.y);
+            pz.add(zk);
         };
         // slot 1 pairs with slot 0 (pair 0); then pairs p = 1.. hold slots 2p, 2p+1
         {
@@ -344,7 +299,7 @@ __global__ void k_moments_real(const float2* __restrict__ psi, const float2* __r
         }
         const float2 z0 = psi[g];
         const double cl = (double)z0.x * z0.x + (double)z0.y * z0.y;
-        const double m2d = m2.value() * inv_ns, prd = pr.value() * inv_ns, pid = pi.value() * inv_ns;
+        const double m2d = m2.value() * inv_ns, prd = pz.x() * inv_ns, pid = pz.y() * inv_ns;
         const double rm = m2d - weyl;
         if (rho_mean) rho_mean[g] = rm;
         if (psi_mean) {

@@ -16,6 +16,7 @@
 // line in `buf`; a missing partner (odd slot count) contributes zero density.
 #pragma once
 #include "fft_engine.cuh"
+#include "pairsum.cuh"
 
 namespace twa {
 
@@ -552,7 +553,9 @@ k_line(const PassArgs a) {
 //   PL_KICK_DRIFT : per slot of the pair: kick with the real Poisson field, drift_x (rows), drift_y
 //   PL_POISSON    : Poisson field plane at fixed k_z: FFT_x (rows), FFT_y, 1/k^2, iFFT_y (columns),
 //                   iFFT_x (rows)
-enum PlaneOp : int { PL_KICK_DRIFT = 0, PL_POISSON = 1, PL_COUNT };
+//   PL_KICK_FWD   : per slot of the pair, into out: kick with the real Poisson field (if a.kick), FFT_x,
+//                   FFT_y (moments; not one of the profiled passes: the profiler takes the axes one by one)
+enum PlaneOp : int { PL_KICK_DRIFT = 0, PL_POISSON = 1, PL_COUNT, PL_KICK_FWD = PL_COUNT };
 
 template <int N, int L, int POP>
 __global__ void __launch_bounds__(L * Plan<N>::T, min_ctas(L * Plan<N>::T))
@@ -630,6 +633,44 @@ k_plane(const PassArgs a) {
             }
             __syncthreads();
         }
+    } else if constexpr (POP == PL_KICK_FWD) {
+        const float2* Wp = a.buf + (long long)f * a.cells + plane;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int slot = 2 * f + h;
+            if (slot >= a.n_slots) break;
+            const float2* F = a.psi + (long long)slot * a.cells + plane;
+            float2* O = a.out + (long long)slot * a.cells + plane;
+            float2* smr = smem + lr * LSR;
+#pragma unroll 1
+            for (int r0 = 0; r0 < N; r0 += L) {
+                const int row = (r0 + lr) * N;
+                const float* Wh = reinterpret_cast<const float*>(Wp) + h;
+#pragma unroll
+                for (int i = 0; i < RMAX; ++i) v[i] = __ldcg(&F[row + pos_nat<N>(tr, i)]);
+                if (a.kick != 0.f) {
+                    float w[RMAX];
+#pragma unroll
+                    for (int i = 0; i < RMAX; ++i) w[i] = __ldcg(&Wh[2 * (row + pos_nat<N>(tr, i))]);
+                    kick_all(v, a.kick, a.kick_lo, [&](int i) { return w[i]; });
+                }
+                fft_line<N, false, WARP, MASK>(v, tr, smr, tw);
+#pragma unroll
+                for (int i = 0; i < RMAX; ++i) O[row + pos_spec<N>(tr, i)] = v[i];
+            }
+            __syncthreads();
+            float2* smc = smem + lc * LSC;
+#pragma unroll 1
+            for (int c0 = 0; c0 < N; c0 += L) {
+                const int col = c0 + lc;
+#pragma unroll
+                for (int i = 0; i < RMAX; ++i) v[i] = __ldcg(&O[col + pos_nat<N>(tc, i) * N]);
+                fft_line<N, false, false>(v, tc, smc, tw);
+#pragma unroll
+                for (int i = 0; i < RMAX; ++i) O[col + pos_spec<N>(tc, i) * N] = v[i];
+            }
+            __syncthreads();
+        }
     } else {
         float2* Wp = a.buf + (long long)f * a.cells + plane;
         float2* smr = smem + lr * LSR;
@@ -667,6 +708,79 @@ k_plane(const PassArgs a) {
         }
     }
 }
+
+// ---------------------------------------------------------------------------------------------
+// Last axis of the mode moments (a_k = sqrt(n dV / M) FFT(psi)_k): forward transform of the column lines of
+// every slot of `buf` (spectral along the other axes), with sum |F|^2 and sum |F|^4 over the slots kept in
+// registers (in slot order, so the sums are those of k_moments_modes bit for bit), and the moments of the
+// CTA's modes formed at the end: the spectra are neither written nor read again.  Per CTA the sum of its
+// modes' <n_k> goes to part.  Bound by reading the batch once and by the last wave (1024 CTAs of 16
+// lines at 128^3, 608 resident): 128^3 x 257 1.2 ms, where the transform pass and the moment pass of its
+// spectra took 2.04.
+struct ModesArgs {
+    double anorm2, inv_ns;
+    double *nk_mean, *nk_var, *nk_cl, *part;
+};
+template <int N, int LINES>
+__global__ void __launch_bounds__(LINES * Plan<N>::T, LINES * Plan<N>::T <= 128 ? 4 : 1)
+k_line_modes(const PassArgs a, const ModesArgs m) {
+    using P = Plan<N>;
+    constexpr int RMAX = P::RMAX, LS = line_stride(N, LINES), NTH = LINES * P::T;
+    extern __shared__ float2 smem[];
+    __shared__ double red[NTH];
+    const int l = threadIdx.x % LINES, t = threadIdx.x / LINES;
+    float2* sm = smem + l * LS;
+    const int q = (int)blockIdx.x * LINES + l;   // the last axis: one outer index
+    const bool act = q < a.Qn;
+    const int base = act ? q : a.Qn - 1;
+    const int S = a.S;
+    float2 v[RMAX];
+    auto transform = [&](const float2* F) {
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) v[i] = __ldcg(&F[base + pos_nat<N>(t, i) * S]);
+        fft_line<N, false, false>(v, t, sm, a.tw);
+    };
+    if (m.nk_cl) {
+        transform(a.buf);
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i)
+                m.nk_cl[base + pos_spec<N>(t, i) * S] = m.anorm2 * ((double)v[i].x * v[i].x + (double)v[i].y * v[i].y);
+        }
+    }
+    DF2 acc[RMAX];
+#pragma unroll 1
+    for (int s = 1; s < a.n_slots; ++s) {
+        transform(a.buf + (long long)s * a.cells);
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) acc[i].add_with_square(fmaf(v[i].x, v[i].x, v[i].y * v[i].y));
+    }
+    double sum = 0.0;
+    if (act) {
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) {
+            const double m2 = m.anorm2 * acc[i].x() * m.inv_ns, m4 = m.anorm2 * m.anorm2 * acc[i].y() * m.inv_ns;
+            const double nk = m2 - 0.5;
+            const int k = base + pos_spec<N>(t, i) * S;
+            if (m.nk_mean) m.nk_mean[k] = nk;
+            if (m.nk_var) m.nk_var[k] = m4 - m2 - nk * nk;
+            sum += nk;
+        }
+    }
+    red[threadIdx.x] = sum;
+    __syncthreads();
+    for (int h = NTH / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        m.part[2 * blockIdx.x] = red[0];
+        m.part[2 * blockIdx.x + 1] = 0.0;
+    }
+}
+
+template <int N>
+int launch_line_modes(const PassArgs& a, const ModesArgs& m, int tiles, cudaStream_t st);
 
 template <int N>
 int launch_plane(int pop, int lines, dim3 grid, const PassArgs& a, cudaStream_t st, bool prepare_only);
