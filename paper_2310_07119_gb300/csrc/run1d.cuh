@@ -28,6 +28,37 @@ struct Run1DArgs {
 // potential.  Both lines form the packed density (each takes the partner's |psi|^2 at the same
 // positions, by a shuffle or through shared memory) and transform it, so each has the potential
 // without a second exchange; the arithmetic of every field is that of the per-interval passes.
+//
+// The run is a serial chain (per step four transforms, each two butterflies deep), so what counts is the
+// latency of one warp, not throughput: a launch of few pairs takes one warp per CTA, which spreads the
+// pairs over the SMs, and the constants of the chain stay in registers for the whole run: 1/k^2, and for
+// lengths of two equal radices (64, 256), whose two stage orders have the same twiddles, those too.
+// 256 cells x 32 streams, 1000 steps: 3.49 ms with the tables read from L1 and eight lines a CTA;
+// 3.11 ms now.
+template <int N>
+__host__ __device__ constexpr bool run1d_reg_tw() {
+    return Plan<N>::S == 2 && Plan<N>::R[0] == Plan<N>::R[1];
+}
+
+// fft_line of such a length with the twiddles W^(r t) of its second stage in registers.
+template <int N, bool INV, unsigned MASK>
+__device__ __forceinline__ void fft_line_reg(float2 (&v)[Plan<N>::RMAX], int t, float2* sm,
+                                             const float4 (&w)[Plan<N>::RMAX - 1]) {
+    constexpr int R = Plan<N>::RMAX;
+    dft<R, INV>(v);
+#pragma unroll
+    for (int r = 0; r < R; ++r) sm[pad_n(N, t * R + r)] = v[r];
+    __syncwarp(MASK);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = sm[pad_n(N, t + r * R)];
+    __syncwarp(MASK);
+#pragma unroll
+    for (int r = 1; r < R; ++r)
+        v[r] = INV ? cmul_c(v[r], make_float2(w[r - 1].x, -w[r - 1].y), make_float2(w[r - 1].z, -w[r - 1].w))
+                   : cmul_c(v[r], make_float2(w[r - 1].x, w[r - 1].y), make_float2(w[r - 1].z, w[r - 1].w));
+    dft<R, INV>(v);
+}
+
 template <int N, int LINES>
 __global__ void __launch_bounds__(LINES * Plan<N>::T, 1)
 k_run1d(const Run1DArgs r) {
@@ -71,14 +102,32 @@ k_run1d(const Run1DArgs r) {
             __syncthreads();  // before the next transform reuses the regions
         }
     };
+    constexpr bool REG = run1d_reg_tw<N>();
+    float4 wr[RMAX - 1];
+    if constexpr (REG) {
+        // entry (r, k = t) of the second stage
+#pragma unroll
+        for (int i = 1; i < RMAX; ++i) wr[i - 1] = __ldg(&tw[tw_offset<N, false, 1>() + (i - 1) * RMAX + t]);
+    }
+    float ik2[RMAX];
+#pragma unroll
+    for (int i = 0; i < RMAX; ++i) ik2[i] = inv_k2(__ldg(&a.k2x[pos_spec<N>(t, i)]));
+    auto fwd = [&](float2 (&x)[RMAX]) {
+        if constexpr (REG) fft_line_reg<N, false, MASK>(x, t, sm, wr);
+        else fft_line<N, false, WARP, MASK>(x, t, sm, tw);
+    };
+    auto inv = [&](float2 (&x)[RMAX]) {
+        if constexpr (REG) fft_line_reg<N, true, MASK>(x, t, sm, wr);
+        else fft_line<N, true, WARP, MASK>(x, t, sm, tw);
+    };
     auto drift = [&]() {
-        fft_line<N, false, WARP, MASK>(v, t, sm, tw);
+        fwd(v);
 #pragma unroll
         for (int i = 0; i < RMAX; ++i) {
             const float4 ph = __ldg(&a.ph[pos_spec<N>(t, i)]);
             v[i] = cmul_c(v[i], make_float2(ph.x, ph.y), make_float2(ph.z, ph.w));
         }
-        fft_line<N, true, WARP, MASK>(v, t, sm, tw);
+        inv(v);
     };
     // packed potential of the pair: W = iFFT(FFT(|psi_0|^2 + i |psi_1|^2) / k^2), on both lines
     auto poisson = [&]() {
@@ -88,13 +137,10 @@ k_run1d(const Run1DArgs r) {
         swap_f(d, e);
 #pragma unroll
         for (int i = 0; i < RMAX; ++i) w[i] = fld ? make_float2(e[i], d[i]) : make_float2(d[i], e[i]);
-        fft_line<N, false, WARP, MASK>(w, t, sm, tw);
+        fwd(w);
 #pragma unroll
-        for (int i = 0; i < RMAX; ++i) {
-            const float m = inv_k2(__ldg(&a.k2x[pos_spec<N>(t, i)]));
-            w[i] = make_float2(w[i].x * m, w[i].y * m);
-        }
-        fft_line<N, true, WARP, MASK>(w, t, sm, tw);
+        for (int i = 0; i < RMAX; ++i) w[i] = make_float2(w[i].x * ik2[i], w[i].y * ik2[i]);
+        inv(w);
     };
     auto pot = [&](int i) { return fld ? w[i].y : w[i].x; };
     // per-cell sums of the pair at output o (the line of field 0 stores them); the pending half kick
