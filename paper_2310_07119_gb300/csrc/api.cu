@@ -986,7 +986,7 @@ int moments_f64(twa_handle* h, Inst& I, double2* psi, const twa_moments_out* o, 
 // and for 1D instances the partial sums of as many outputs as fit 16 MB (none when two do not).
 int alloc_f64(twa_handle* h, Inst& I) {
     const double field = (double)I.cells * sizeof(double2);
-    const int most = (int)std::max(1.0, std::min(32768.0, (double)(1LL << 30) / field));
+    const int most = (int)std::max(1.0, std::min(32767.0, (double)(1LL << 30) / field));
     if (I.mode != MODE_1D) {
         I.w_pairs = std::min(I.n_pairs, most);
         while (dalloc(h, &I.work64, (size_t)I.w_pairs * I.cells) != 0) {  // fewer at a time when memory is short

@@ -709,6 +709,105 @@ k_plane(const PassArgs a) {
     }
 }
 
+// The same passes of planes up to 64 x 64 with the plane in shared memory between its axes: one CTA
+// transforms one plane of one slot (PL_POISSON: of one pair's Poisson field), which is read and written
+// once.  Small fields are bound by latency: a plane written back and read through L2 between the axes,
+// and the two slots of a pair one after the other, took most of a launch (32^3 x 65: PL_KICK_DRIFT 28 us,
+// PL_POISSON 17; now 23 and 13; 64^3 x 257 418 -> 396 and 197 -> 167).  Rows are padded by one element for the column accesses.
+template <int N, int L, int POP>
+__global__ void __launch_bounds__(L * Plan<N>::T, min_ctas(L * Plan<N>::T))
+k_plane_s(const PassArgs a) {
+    using P = Plan<N>;
+    constexpr int T = P::T, RMAX = P::RMAX, LD = N + 1;
+    constexpr int LSR = line_stride_rows(N, T), LSC = line_stride(N, L);
+    constexpr bool WARP = (T <= 32);
+    constexpr unsigned MASK = (L * T >= 32) ? 0xffffffffu : ((1u << (L * T)) - 1u);
+    extern __shared__ float2 smem[];
+    float2* pl = smem + (L * LSR > L * LSC ? L * LSR : L * LSC);   // [row][LD]
+    const int tid = threadIdx.x;
+    const int lr = tid / T, tr = tid % T, lc = tid % L, tc = tid / L;
+    const float4* __restrict__ tw = a.tw;
+    const long long plane = (long long)blockIdx.x * N * N;
+    float2* smr = smem + lr * LSR;
+    float2* smc = smem + lc * LSC;
+    float2 v[RMAX];
+    auto phase = [&](const float4* ph, int t) {
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) {
+            const float4 p = __ldg(&ph[pos_spec<N>(t, i)]);
+            v[i] = cmul_c(v[i], make_float2(p.x, p.y), make_float2(p.z, p.w));
+        }
+    };
+    // pair blockIdx.y of the Poisson field, or slot 2 blockIdx.y + blockIdx.z
+    const int slot = 2 * blockIdx.y + blockIdx.z;
+    if (POP != PL_POISSON && slot >= a.n_slots) return;
+    const float2* F = POP == PL_POISSON ? a.buf + (long long)blockIdx.y * a.cells + plane
+                                        : a.psi + (long long)slot * a.cells + plane;
+    float2* O = POP == PL_POISSON ? a.buf + (long long)blockIdx.y * a.cells + plane
+                                  : (POP == PL_KICK_FWD ? a.out : a.psi) + (long long)slot * a.cells + plane;
+    const float* Wh = reinterpret_cast<const float*>(a.buf + (long long)blockIdx.y * a.cells + plane) + blockIdx.z;
+#pragma unroll 1
+    for (int r0 = 0; r0 < N; r0 += L) {
+        const int row = r0 + lr;
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) v[i] = __ldcg(&F[row * N + pos_nat<N>(tr, i)]);
+        if (POP == PL_KICK_DRIFT || (POP == PL_KICK_FWD && a.kick != 0.f)) {
+            float w[RMAX];
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) w[i] = __ldcg(&Wh[2 * (row * N + pos_nat<N>(tr, i))]);
+            kick_all(v, a.kick, a.kick_lo, [&](int i) { return w[i]; });
+        }
+        fft_line<N, false, WARP, MASK>(v, tr, smr, tw);
+        if constexpr (POP == PL_KICK_DRIFT) {
+            phase(a.ph, tr);
+            fft_line<N, true, WARP, MASK>(v, tr, smr, tw);
+        }
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i)
+            pl[row * LD + (POP == PL_KICK_DRIFT ? pos_nat<N>(tr, i) : pos_spec<N>(tr, i))] = v[i];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int c0 = 0; c0 < N; c0 += L) {
+        const int col = c0 + lc;
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) v[i] = pl[pos_nat<N>(tc, i) * LD + col];
+        fft_line<N, false, false>(v, tc, smc, tw);
+        if constexpr (POP == PL_KICK_FWD) {
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) O[col + pos_spec<N>(tc, i) * N] = v[i];
+        } else if constexpr (POP == PL_KICK_DRIFT) {
+            phase(a.ph2, tc);
+            fft_line<N, true, false>(v, tc, smc, tw);
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) O[col + pos_nat<N>(tc, i) * N] = v[i];
+        } else {
+            // k_x (the column) and k_z (the plane) are fixed, k_y is read per value
+            const float k2f = __ldg(&a.k2x[col]) + __ldg(&a.k2z[blockIdx.x]);
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) {
+                const float m = inv_k2(k2f + __ldg(&a.k2y[pos_spec<N>(tc, i)]));
+                v[i] = make_float2(v[i].x * m, v[i].y * m);
+            }
+            fft_line<N, true, false>(v, tc, smc, tw);
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) pl[pos_nat<N>(tc, i) * LD + col] = v[i];
+        }
+    }
+    if constexpr (POP == PL_POISSON) {
+        __syncthreads();
+#pragma unroll 1
+        for (int r0 = 0; r0 < N; r0 += L) {
+            const int row = r0 + lr;
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) v[i] = pl[row * LD + pos_spec<N>(tr, i)];
+            fft_line<N, true, WARP, MASK>(v, tr, smr, tw);
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) O[row * N + pos_nat<N>(tr, i)] = v[i];
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Last axis of the mode moments (a_k = sqrt(n dV / M) FFT(psi)_k): forward transform of the column lines of
 // every slot of `buf` (spectral along the other axes), with sum |F|^2 and sum |F|^4 over the slots kept in
