@@ -13,8 +13,9 @@
 //     idle: 100 steps of 32 streams of 256 cells took 25,000 launches and 186 ms.
 //   * A 1D field stays on one SM for a whole run (k64_run1d), a stream per CTA.
 // Measured before and after (one GB300): 100 steps of 32 streams of 256 cells, moments every 10,
-// 182.6 -> 1.55 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.19 ms, where FP64 issue
-// alone (about 245 instructions per value and step at 2 per cycle and SM) takes 3.9 ms.
+// 182.6 -> 1.04 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.18 ms.  A warp's FP64
+// instruction occupies its scheduler's unit for about 100 cycles whatever its active lanes (from the times
+// of 8 to 2048 cells), which is what is left in both.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
@@ -38,78 +39,71 @@ __device__ __forceinline__ void bfly1(double2& a, double2& b) {
     b = d;
 }
 
+// Radix-4 butterfly with twiddles w1, w2 = w1^2 (conjugated by the caller for an inverse), outputs in order.
+template <bool TW>
+__device__ __forceinline__ void radix4(double2 (&v)[4], double2 w1, double2 w2, bool inv) {
+    if constexpr (TW) {
+        bfly(v[0], v[2], w2);
+        bfly(v[1], v[3], w2);
+        bfly(v[0], v[1], w1);
+        bfly(v[2], v[3], inv ? make_double2(-w1.y, w1.x) : make_double2(w1.y, -w1.x));
+    } else {
+        bfly1(v[0], v[2]);
+        bfly1(v[1], v[3]);
+        v[3] = inv ? make_double2(-v[3].y, v[3].x) : make_double2(v[3].y, -v[3].x);
+        bfly1(v[0], v[1]);
+        bfly1(v[2], v[3]);
+    }
+    // v = outputs 0, 2, 1, 3
+    const double2 t = v[1];
+    v[1] = v[2];
+    v[2] = t;
+}
+
 // Shared-memory slot of element i: one 16-byte slot of padding per 8 (the first stages store with
 // strides of two and four elements).
 __device__ __forceinline__ int pad64(int i) { return i + (i >> 3); }
 __host__ __device__ constexpr int line64(int n) { return n + n / 8 + 1; }
 
-// Transform of one line of N = 2^lg values by N / V threads: thread j holds elements j + r N / V, r < V,
+// Transform of one line of N = 2^lg values by N / 4 threads: thread j holds elements j + r N / 4, r < 4,
 // before and after.  a and b: two exchange lines of line64(N), used in turn by every exchange of a kernel
 // (a line is written again only behind the barrier of the exchange in between, so each exchange has
 // one barrier); every thread of the CTA takes part.
-template <int V>
-__device__ __forceinline__ void fft64(double2 (&v)[V], int j, int N, int lg, bool inv, double2*& a, double2*& b,
+__device__ __forceinline__ void fft64(double2 (&v)[4], int j, int N, int lg, bool inv, double2*& a, double2*& b,
                                       const double2* __restrict__ tw) {
     auto root = [&](int e) {
         double2 w = __ldg(&tw[e]);
         if (inv) w.y = -w.y;
         return w;
     };
-    auto exchange = [&](const int (&d)[V]) {
-#pragma unroll
-        for (int r = 0; r < V; ++r) a[pad64(d[r])] = v[r];
+    const int q = N / 4;
+    auto exchange = [&](int d0, int d1, int d2, int d3) {
+        a[pad64(d0)] = v[0];
+        a[pad64(d1)] = v[1];
+        a[pad64(d2)] = v[2];
+        a[pad64(d3)] = v[3];
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < V; ++r) v[r] = a[pad64(j + r * (N / V))];
+        for (int r = 0; r < 4; ++r) v[r] = a[pad64(j + r * q)];
         double2* t = a;
         a = b;
         b = t;
     };
-    int ns = 1;
-    if constexpr (V == 2) {
+    int ls = 0;  // log2 of the sub-transform length ns
+    if (lg & 1) {  // radix 2: the butterflies j and j + N / 4
+        bfly1(v[0], v[2]);
+        bfly1(v[1], v[3]);
+        exchange(2 * j, 2 * (j + q), 2 * j + 1, 2 * (j + q) + 1);
+        ls = 1;
+    }
 #pragma unroll 1
-        for (; ns < N; ns *= 2) {
-            const int k = j & (ns - 1);
-            if (ns == 1) bfly1(v[0], v[1]);
-            else bfly(v[0], v[1], root(k * (N / (2 * ns))));
-            if (2 * ns < N) {
-                const int d = (j - k) * 2 + k;
-                exchange({d, d + ns});
-            }
-        }
-    } else {
-        const int q = N / 4;
-        if (lg & 1) {  // radix 2: the butterflies j and j + N / 4
-            bfly1(v[0], v[2]);
-            bfly1(v[1], v[3]);
-            exchange({2 * j, 2 * (j + q), 2 * j + 1, 2 * (j + q) + 1});
-            ns = 2;
-        }
-#pragma unroll 1
-        for (; ns < N; ns *= 4) {
-            const int k = j & (ns - 1), s = q / ns;
-            if (ns == 1) {
-                bfly1(v[0], v[2]);
-                bfly1(v[1], v[3]);
-                const double2 n = inv ? make_double2(-v[3].y, v[3].x) : make_double2(v[3].y, -v[3].x);
-                v[3] = n;
-                bfly1(v[0], v[1]);
-                bfly1(v[2], v[3]);
-            } else {
-                const double2 w1 = root(k * s), w2 = root(2 * k * s);
-                bfly(v[0], v[2], w2);
-                bfly(v[1], v[3], w2);
-                bfly(v[0], v[1], w1);
-                bfly(v[2], v[3], inv ? make_double2(-w1.y, w1.x) : make_double2(w1.y, -w1.x));
-            }
-            // v = outputs 0, 2, 1, 3 of the butterfly
-            const double2 t = v[1];
-            v[1] = v[2];
-            v[2] = t;
-            if (4 * ns < N) {
-                const int d = (j - k) * 4 + k;
-                exchange({d, d + ns, d + 2 * ns, d + 3 * ns});
-            }
+    for (; ls < lg; ls += 2) {
+        const int ns = 1 << ls, k = j & (ns - 1);
+        if (ls == 0) radix4<false>(v, make_double2(1.0, 0.0), make_double2(1.0, 0.0), inv);
+        else radix4<true>(v, root(k << (lg - 2 - ls)), root(k << (lg - 1 - ls)), inv);
+        if (ls + 2 < lg) {
+            const int d = (j - k) * 4 + k;
+            exchange(d, d + ns, d + 2 * ns, d + 3 * ns);
         }
     }
 }
@@ -173,7 +167,7 @@ __device__ __forceinline__ void store4(const double2 (&v)[4], double2* f, const 
     for (int r = 0; r < 4; ++r) f[l.at + (long long)r * l.step] = v[r];
 }
 __device__ __forceinline__ void fft4(double2 (&v)[4], Line64& l, const Axis64& x, bool inv) {
-    fft64<4>(v, l.j, x.N, x.lg, inv, l.a, l.b, x.tw);
+    fft64(v, l.j, x.N, x.lg, inv, l.a, l.b, x.tw);
 }
 __device__ __forceinline__ void drift4(double2 (&v)[4], Line64& l, const Axis64& x) {
     fft4(v, l, x, false);
@@ -263,19 +257,87 @@ __global__ void __launch_bounds__(512) k64_field(Axis64 x, const double2* src, d
     store4(v, dst + (long long)blockIdx.y * x.cells, l);
 }
 
+// One line of 2^LG values for a whole run: V values per thread (2: radix 2; 4: radix 4 with a radix-2 stage
+// first when LG is odd), its twiddles in registers.  An exchange of up to 32 threads needs no CTA barrier.
+template <int LG, int V>
+struct Line1D {
+    static constexpr int N = 1 << LG, TH = N / V;
+    static constexpr int FIRST = V == 4 && (LG & 1);               // radix-2 stage before the radix-4 ones
+    static constexpr int STEP = V == 2 ? 1 : 2;                     // levels per stage
+    static constexpr int STAGES = (LG - FIRST) / STEP;
+    static constexpr int NTW = V == 2 ? STAGES : 2 * STAGES;
+    double2 w[NTW];
+    double2 *a, *b;
+    int j;
+    __device__ __forceinline__ void init(int j_, double2* sm, const double2* __restrict__ tw) {
+        j = j_;
+        a = sm;
+        b = sm + line64(N);
+#pragma unroll
+        for (int s = 0; s < STAGES; ++s) {
+            const int ls = FIRST + s * STEP, k = j & ((1 << ls) - 1);
+            if constexpr (V == 2) {
+                w[s] = tw[k << (LG - 1 - ls)];
+            } else {
+                w[2 * s] = tw[k << (LG - 2 - ls)];
+                w[2 * s + 1] = tw[k << (LG - 1 - ls)];
+            }
+        }
+    }
+    __device__ __forceinline__ void exchange(double2 (&v)[V], const int (&d)[V]) {
+#pragma unroll
+        for (int r = 0; r < V; ++r) a[pad64(d[r])] = v[r];
+        if constexpr (TH <= 32) __syncwarp(TH == 32 ? 0xffffffffu : (1u << (TH & 31)) - 1u);
+        else __syncthreads();
+#pragma unroll
+        for (int r = 0; r < V; ++r) v[r] = a[pad64(j + r * TH)];
+        double2* t = a;
+        a = b;
+        b = t;
+    }
+    template <bool INV>
+    __device__ __forceinline__ void transform(double2 (&v)[V]) {
+        auto root = [&](int i) { return INV ? make_double2(w[i].x, -w[i].y) : w[i]; };
+        if constexpr (FIRST) {
+            bfly1(v[0], v[2]);
+            bfly1(v[1], v[3]);
+            exchange(v, {2 * j, 2 * (j + TH), 2 * j + 1, 2 * (j + TH) + 1});
+        }
+#pragma unroll
+        for (int s = 0; s < STAGES; ++s) {
+            const int ls = FIRST + s * STEP, ns = 1 << ls, k = j & (ns - 1);
+            if constexpr (V == 2) {
+                if (s == 0) bfly1(v[0], v[1]);
+                else bfly(v[0], v[1], root(s));
+                const int d = (j - k) * 2 + k;
+                if (s + 1 < STAGES) exchange(v, {d, d + ns});
+            } else {
+                if (ls == 0) radix4<false>(v, w[0], w[0], INV);
+                else radix4<true>(v, root(2 * s), root(2 * s + 1), INV);
+                const int d = (j - k) * 4 + k;
+                if (s + 1 < STAGES) exchange(v, {d, d + ns, d + 2 * ns, d + 3 * ns});
+            }
+        }
+    }
+};
+
 // A whole 1D run of one stream (slot blockIdx.x) on one SM: KDK steps with adjacent half kicks merged,
 // and at the start and after every out_every steps the synchronized field's |psi|^2, Re psi and Im psi
 // per cell (the classical slot: |psi|^2) into partial sums that k_finish_run1d adds over the streams.
-// FP64 issue bounds it (about 9 us a step at 256 cells; N / 2 threads up to 256 cells so that the four
-// schedulers of the SM all have a warp), and an exchange costs a barrier of a few warps.
-template <int V>
-__global__ void __launch_bounds__(512) k64_run1d(double2* psi, int N, int lg, const double2* __restrict__ tw,
-                                                 const double2* __restrict__ ph, const double* __restrict__ k2, double mulc,
-                                                 double kick, int n_out, int out_every, int n_real, double* part,
-                                                 double* part_cl, double* part_bad) {
+// Bound by FP64 issue per scheduler, so up to 256 cells two values per thread keep all four schedulers
+// at work (256 x 32: 17.5 us a step against 19.9 with four); batches that fill them anyway take four
+// (256 x 500: 41 us against 63).  Twiddles and multipliers stay in
+// registers and the length is a template parameter: 100 steps of 32 streams of 256 cells 1.55 -> 1.04 ms.
+template <int LG, int V>
+__global__ void __launch_bounds__((1 << LG) / V) k64_run1d(double2* psi, const double2* __restrict__ tw,
+                                                           const double2* __restrict__ ph, const double* __restrict__ k2,
+                                                           double mulc, double kick, int n_out, int out_every, int n_real,
+                                                           double* part, double* part_cl, double* part_bad) {
+    constexpr int N = 1 << LG;
     extern __shared__ double2 sm64[];
-    double2 *a = sm64, *b = sm64 + line64(N);
     const int j = threadIdx.x, q = N / V, slot = blockIdx.x;
+    Line1D<LG, V> ln;
+    ln.init(j, sm64, tw);
     double2* f = psi + (long long)slot * N;
     double2 v[V], p[V];
     double m[V], pot[V];
@@ -290,10 +352,10 @@ __global__ void __launch_bounds__(512) k64_run1d(double2* psi, int N, int lg, co
         double2 w[V];
 #pragma unroll
         for (int r = 0; r < V; ++r) w[r] = make_double2(fma(v[r].x, v[r].x, v[r].y * v[r].y), 0.0);
-        fft64<V>(w, j, N, lg, false, a, b, tw);
+        ln.template transform<false>(w);
 #pragma unroll
         for (int r = 0; r < V; ++r) w[r] = make_double2(w[r].x * m[r], w[r].y * m[r]);
-        fft64<V>(w, j, N, lg, true, a, b, tw);
+        ln.template transform<true>(w);
 #pragma unroll
         for (int r = 0; r < V; ++r) pot[r] = w[r].x;
     };
@@ -329,10 +391,10 @@ __global__ void __launch_bounds__(512) k64_run1d(double2* psi, int N, int lg, co
             const double kk = (o == 1 && s == 0) ? 0.5 * kick : kick;
 #pragma unroll
             for (int r = 0; r < V; ++r) v[r] = kick64(v[r], kk * pot[r]);
-            fft64<V>(v, j, N, lg, false, a, b, tw);
+            ln.template transform<false>(v);
 #pragma unroll
             for (int r = 0; r < V; ++r) v[r] = zmul(v[r], p[r]);
-            fft64<V>(v, j, N, lg, true, a, b, tw);
+            ln.template transform<true>(v);
             poisson();
         }
         output(o, 0.5 * kick);
@@ -455,8 +517,7 @@ int prepare64() {
     for (const void* k : {(const void*)k64_kick_drift, (const void*)k64_drift, (const void*)k64_drift_rho,
                           (const void*)k64_field})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
-    for (const void* k : {(const void*)k64_run1d<2>, (const void*)k64_run1d<4>})
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
+    if (cudaFuncSetAttribute(k64_run1d<11, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
     return 0;
 }
 
@@ -520,14 +581,24 @@ int launch_f64_steps(double2* psi, double2* W, int w_pairs, int n_slots, const G
 
 int launch_f64_run1d(double2* psi, int n_slots, const Geom64& g, const Tables64& t, double mulc, double kick, int n_out,
                      int out_every, double* part, double* part_cl, double* part_bad, cudaStream_t st, long long* nl) {
-    const int N = g.n[0], lg = ilog2(N);
-    const size_t sm = 2 * (size_t)line64(N) * sizeof(double2);
-    if (N <= 256)
-        k64_run1d<2><<<n_slots, N / 2, sm, st>>>(psi, N, lg, t.tw[0], t.ph[0], t.k2[0], mulc, kick, n_out, out_every,
-                                                 n_slots - 1, part, part_cl, part_bad);
-    else
-        k64_run1d<4><<<n_slots, N / 4, sm, st>>>(psi, N, lg, t.tw[0], t.ph[0], t.k2[0], mulc, kick, n_out, out_every,
-                                                 n_slots - 1, part, part_cl, part_bad);
+    auto go = [&](auto kernel, int threads) {
+        const size_t sm = 2 * (size_t)line64(g.n[0]) * sizeof(double2);
+        kernel<<<n_slots, threads, sm, st>>>(psi, t.tw[0], t.ph[0], t.k2[0], mulc, kick, n_out, out_every, n_slots - 1,
+                                             part, part_cl, part_bad);
+    };
+    // from two CTAs per SM on the FP64 units are busy without the second warp of a value pair
+    const bool many = n_slots > 2 * 152;
+    switch (g.n[0]) {
+        case 8: go(k64_run1d<3, 2>, 4); break;
+        case 16: go(k64_run1d<4, 2>, 8); break;
+        case 32: go(k64_run1d<5, 2>, 16); break;
+        case 64: go(k64_run1d<6, 2>, 32); break;
+        case 128: many ? go(k64_run1d<7, 4>, 32) : go(k64_run1d<7, 2>, 64); break;
+        case 256: many ? go(k64_run1d<8, 4>, 64) : go(k64_run1d<8, 2>, 128); break;
+        case 512: go(k64_run1d<9, 4>, 128); break;
+        case 1024: go(k64_run1d<10, 4>, 256); break;
+        default: go(k64_run1d<11, 4>, 512); break;
+    }
     ++*nl;
     return 0;
 }
