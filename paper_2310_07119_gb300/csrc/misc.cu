@@ -69,9 +69,9 @@ __device__ const WignerTables g_wigner = make_wigner_tables();
 
 // The same for float fields: the normals in pairs of floats (wigner.cuh) instead of FP64, each value
 // rounded to float once from about 2^-37.  A thread draws up to `spt` consecutive slots of one cell
-// (cells = 2^lc), so the cell's classical value is split into floats once per spt streams.  Bound by
-// FP32 issue (about 250 instructions a value, Philox a third of them); drawing 128^3 x 64 streams took
-// 19.07 ms in FP64 and takes 1.09 ms (its write alone 0.16 ms), with the same
+// (cells = 2^lc), two at a time, so the cell's classical value is split into floats once per spt streams.
+// Bound by the integer and FP32 units (Philox a third of the work); drawing 128^3 x 64 streams took
+// 19.07 ms in FP64, 1.09 ms one value at a time and takes 0.93 to 1.0 ms (its write alone 0.16 ms), with the same
 // error against FP64 (2.5e-8, the rounding).
 __global__ void __launch_bounds__(256)
 k_sample_f32(const double2* __restrict__ psi_cl, float2* __restrict__ psi, int lc, int n_slots, int spt, uint32_t k0,
@@ -88,27 +88,30 @@ k_sample_f32(const double2* __restrict__ psi_cl, float2* __restrict__ psi, int l
     if (first >= n_slots) return;
     const int last = (int)min((long long)n_slots, first + spt);
     const double2 zc = psi_cl[g];
-    F2 cx{(float)zc.x, 0.f}, cy{(float)zc.y, 0.f};
+    const float hx = (float)zc.x, hy = (float)zc.y;
     // the remainder of a value that is no finite float is nothing
-    if (isfinite(cx.hi)) cx.lo = (float)(zc.x - (double)cx.hi);
-    if (isfinite(cy.hi)) cy.lo = (float)(zc.y - (double)cy.hi);
-    const F2 sg{sigma, sigma_lo};
+    const float rx = isfinite(hx) ? (float)(zc.x - (double)hx) : 0.f, ry = isfinite(hy) ? (float)(zc.y - (double)hy) : 0.f;
+    const Pair<float2> cx{make_float2(hx, hx), make_float2(rx, rx)}, cy{make_float2(hy, hy), make_float2(ry, ry)};
+    const Pair<float2> sg{make_float2(sigma, sigma), make_float2(sigma_lo, sigma_lo)};
     float2* out = psi + first * cells + g;
-    for (int s = (int)first; s < last; ++s, out += cells) {
-        float2 z = make_float2(cx.hi, cy.hi);
-        if (s > 0) {
-            uint32_t c0 = (uint32_t)g, c1 = (uint32_t)s, c2 = inst, c3 = 0;
-            philox4x32_10(c0, c1, c2, c3, k0, k1);
-            const F2 r = mul22(sg, bm_radius(c0, tab.rec));
-            F2 co, si;
-            bm_direction(c1, tab.dir, co, si);
-            const F2 nx = mul22(r, co), ny = mul22(r, si);
-            z = make_float2(add22_round(cx, nx), add22_round(cy, ny));
-            // infinities, NaN and overflow: the error terms of the pair sum are no numbers there
-            if (!isfinite(z.x)) z.x = cx.hi + nx.hi;
-            if (!isfinite(z.y)) z.y = cy.hi + ny.hi;
-        }
-        *out = z;
+    // slots s and s + 1 at once, the lanes of every float2
+    for (int s = (int)first; s < last; s += 2, out += 2 * cells) {
+        uint32_t r0 = (uint32_t)g, d0 = (uint32_t)s, t0 = inst, u0 = 0;
+        uint32_t r1 = (uint32_t)g, d1 = (uint32_t)s + 1, t1 = inst, u1 = 0;
+        philox4x32_10(r0, d0, t0, u0, k0, k1);
+        philox4x32_10(r1, d1, t1, u1, k0, k1);
+        const RadiusWord a = radius_word(r0, tab.rec), b = radius_word(r1, tab.rec);
+        const DirectionWord p = direction_word(d0, tab.dir), q = direction_word(d1, tab.dir);
+        const Pair<float2> r = mul22(sg, bm_radius(make_float2(a.mh, b.mh), make_float2(a.ml, b.ml), make_float2(a.T.x, b.T.x),
+                                                   make_float2(a.T.y, b.T.y), make_float2(a.T.z, b.T.z), make_float2(a.E, b.E)));
+        Pair<float2> co, si;
+        bm_direction(make_float2(p.rest, q.rest), make_float2(p.D.x, q.D.x), make_float2(p.D.y, q.D.y),
+                     make_float2(p.D.z, q.D.z), make_float2(p.D.w, q.D.w), co, si);
+        const Pair<float2> nx = mul22(r, co), ny = mul22(r, si);
+        const float2 x = add22_round(cx, nx), y = add22_round(cy, ny);
+        // infinities, NaN and overflow: the error terms of the pair sum are no numbers there; slot 0 is psi_cl
+        out[0] = s == 0 ? make_float2(hx, hy) : make_float2(isfinite(x.x) ? x.x : hx + nx.hi.x, isfinite(y.x) ? y.x : hy + ny.hi.x);
+        if (s + 1 < last) out[cells] = make_float2(isfinite(x.y) ? x.y : hx + nx.hi.y, isfinite(y.y) ? y.y : hy + ny.hi.y);
     }
 }
 

@@ -326,8 +326,8 @@ struct Line1D {
 // per cell (the classical slot: |psi|^2) into partial sums that k_finish_run1d adds over the streams.
 // Bound by FP64 issue per scheduler, so up to 256 cells two values per thread keep all four schedulers
 // at work (256 x 32: 17.5 us a step against 19.9 with four); batches that fill them anyway take four
-// (256 x 500: 41 us against 63).  Twiddles and multipliers stay in
-// registers and the length is a template parameter: 100 steps of 32 streams of 256 cells 1.55 -> 1.04 ms.
+// (256 x 500: 41 us against 63).  Twiddles and multipliers stay in registers and the length is a template
+// parameter: 100 steps of 32 streams of 256 cells 1.55 -> 1.04 ms.
 template <int LG, int V>
 __global__ void __launch_bounds__((1 << LG) / V) k64_run1d(double2* psi, const double2* __restrict__ tw,
                                                            const double2* __restrict__ ph, const double* __restrict__ k2,

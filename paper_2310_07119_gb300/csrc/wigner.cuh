@@ -12,18 +12,22 @@
 //   sqrt    Karp's correction of x rsqrt(x) (Karp and Markstein, ACM TOMS 23, 1997);
 //   angle   2 pi u: the nearest of 256 directions in integers, the rest by the series of sin and cos,
 //           joined by the addition theorems.
-// The functions also compile for the host, so their error can be held without a GPU.
+// The arithmetic is written once for a lane type V: float, also on the host, so that its error can be held
+// without a GPU, and float2 on the GPU, two values at once in packed FP32 (half the issue slots).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
+#include "fft_engine.cuh"
+
 namespace twa {
 
-struct F2 {  // hi + lo
-    float hi, lo;
+template <class V>
+struct Pair {  // hi + lo
+    V hi, lo;
 };
-constexpr F2 split2(double x) { return F2{(float)x, (float)(x - (double)(float)x)}; }
+constexpr Pair<float> split2(double x) { return Pair<float>{(float)x, (float)(x - (double)(float)x)}; }
 
 // Tables, formed at compile time in double and split into float pairs (their remainders below 2^-49).
 struct WignerTables {
@@ -51,8 +55,8 @@ constexpr WignerTables make_wigner_tables() {
         const int q = ((j + 32) / 64) % 4;          // nearest quarter turn
         const double d = pi * (j - 64 * ((j + 32) / 64)) / 128.0;
         const double c = ce_trig(d, false), s = ce_trig(d, true);
-        const F2 a = split2(q == 0 ? c : (q == 1 ? -s : (q == 2 ? -c : s)));
-        const F2 b = split2(q == 0 ? s : (q == 1 ? c : (q == 2 ? -s : -c)));
+        const Pair<float> a = split2(q == 0 ? c : (q == 1 ? -s : (q == 2 ? -c : s)));
+        const Pair<float> b = split2(q == 0 ? s : (q == 1 ? c : (q == 2 ? -s : -c)));
         w.dir[j].x = a.hi;
         w.dir[j].y = a.lo;
         w.dir[j].z = b.hi;
@@ -65,7 +69,7 @@ constexpr WignerTables make_wigner_tables() {
         if (i == 127) k = 128;
         const bool half = i >= 53;                   // 1 + 53 / 128 = sqrt 2
         const double r = k / 256.0;
-        const F2 t = split2(half ? -ce_ln(2.0 * r) : -ce_ln(r));
+        const Pair<float> t = split2(half ? -ce_ln(2.0 * r) : -ce_ln(r));
         w.rec[i].x = (float)r;
         w.rec[i].y = t.hi;
         w.rec[i].z = t.lo;
@@ -74,93 +78,130 @@ constexpr WignerTables make_wigner_tables() {
     return w;
 }
 
+#define TWA_HD __host__ __device__ __forceinline__
 #ifdef __CUDA_ARCH__
 #define TWA_CLZ(x) __clz((int)(x))
-#define TWA_MUL(a, b) __fmul_rn(a, b)  // a product whose rounding error is taken up later: never part of an fma
+// never part of an fma: the rounding errors of these are taken up later
+TWA_HD float vadd(float a, float b) { return __fadd_rn(a, b); }
+TWA_HD float vsub(float a, float b) { return __fsub_rn(a, b); }
+TWA_HD float vmul(float a, float b) { return __fmul_rn(a, b); }
+TWA_HD float vrsqrt(float a) { return rsqrtf(a); }
 #else
 #define TWA_CLZ(x) ((x) ? __builtin_clz(x) : 32)
-#define TWA_MUL(a, b) ((a) * (b))
+TWA_HD float vadd(float a, float b) { return a + b; }
+TWA_HD float vsub(float a, float b) { return a - b; }
+TWA_HD float vmul(float a, float b) { return a * b; }
+TWA_HD float vrsqrt(float a) { return 1.f / sqrtf(a); }
 #endif
+TWA_HD float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return f2_add(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return f2_sub(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return f2_mul(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return f2_fma(a, b, c); }
+__device__ __forceinline__ float2 vrsqrt(float2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+template <class V>
+TWA_HD V vset(float c) {
+    if constexpr (sizeof(V) == sizeof(float)) return c;
+    else return V{c, c};
+}
+TWA_HD float vneg(float a) { return -a; }
+TWA_HD float2 vneg(float2 a) { return float2{-a.x, -a.y}; }
 
 // a + b = s + e exactly (Knuth)
-__host__ __device__ __forceinline__ F2 two_sum(float a, float b) {
-    const float s = a + b, bb = s - a;
-    return F2{s, (a - (s - bb)) + (b - bb)};
+template <class V>
+TWA_HD Pair<V> two_sum(V a, V b) {
+    const V s = vadd(a, b), bb = vsub(s, a);
+    return {s, vadd(vsub(a, vsub(s, bb)), vsub(b, bb))};
 }
 // the same when |a| >= |b| or a = 0 (Dekker)
-__host__ __device__ __forceinline__ F2 fast_two_sum(float a, float b) {
-    const float s = a + b;
-    return F2{s, b - (s - a)};
+template <class V>
+TWA_HD Pair<V> fast_two_sum(V a, V b) {
+    const V s = vadd(a, b);
+    return {s, vsub(b, vsub(s, a))};
 }
 // (a.hi + a.lo) (b.hi + b.lo)
-__host__ __device__ __forceinline__ F2 mul22(F2 a, F2 b) {
-    const float p = TWA_MUL(a.hi, b.hi);
-    return F2{p, fmaf(a.hi, b.hi, -p) + fmaf(a.hi, b.lo, a.lo * b.hi)};
+template <class V>
+TWA_HD Pair<V> mul22(Pair<V> a, Pair<V> b) {
+    const V p = vmul(a.hi, b.hi);
+    return {p, vadd(vfma(a.hi, b.hi, vneg(p)), vfma(a.hi, b.lo, vmul(a.lo, b.hi)))};
 }
 
-// sqrt(-2 ln u), u = (c + 1/2) / 2^32.
-__host__ __device__ __forceinline__ F2 bm_radius(uint32_t c, const float4* rec) {
-    // a = 2 c + 1 = (1 + F / 2^32) 2^e
+// The integer reductions of one word c (u = (c + 1/2) / 2^32), as floats.
+struct RadiusWord {  // u = a / 2^33, a = 2 c + 1 = (1 + F / 2^32) 2^e
+    float mh, ml, E;  // top 24 bits of m and the last 9; e - 33
+    float4 T;         // table entry
+};
+TWA_HD RadiusWord radius_word(uint32_t c, const float4* rec) {
     const int n = 31 - TWA_CLZ(c);                   // -1 for c = 0
     const uint32_t F = c ? (((c << (31 - n)) << 1) | (1u << (31 - n))) : 0u;
-    const float4 T = rec[F >> 25];
-    const float mh = fmaf((float)(F >> 9), 0x1p-23f, 1.f);   // top 24 bits of m, then the last 9
-    const float ml = (float)(F & 511u) * 0x1p-32f;
-    // m r - 1: both terms exact (|f| < 2^-7, r of 8 bits), then ordered
-    const F2 f = two_sum(fmaf(mh, T.x, -1.f), ml * T.x);
-    const float fh = f.hi, fl = f.lo;
-    // log(1 + f) = f - f^2 / 2 + f^3 (1/3 - f/4 + f^2/5 - f^3/6 + f^4/7)
-    const float f2 = TWA_MUL(fh, fh), f2l = fmaf(fh, fh, -f2) + 2.f * fh * fl;
-    const float p = fmaf(fh, fmaf(fh, fmaf(fh, fmaf(fh, 1.f / 7.f, -1.f / 6.f), 0.2f), -0.25f), 1.f / 3.f);
-    const float tail = fmaf(fh * f2, p, fmaf(-0.5f, f2l, fl));
-    const F2 l = fast_two_sum(fh, -0.5f * f2);
-    // ln u = E ln 2 + T + log(1 + f); ln 2 as 15 bits (E ln2_hi is exact) and the rest
-    const float E = (float)(n + 1 - 33) + T.w;
-    const F2 s0 = fast_two_sum(E * 0x1.62e4p-1f, T.y);       // |E ln 2| >= |T| or E = 0
-    const F2 s1 = two_sum(s0.hi, l.hi);
-    const float lo = ((s0.lo + s1.lo) + (l.lo + tail)) + fmaf(E, 0x1.7f7d1cp-20f, T.z);
-    const F2 L = fast_two_sum(s1.hi, lo);
-    const float x = -2.f * L.hi, xl = -2.f * L.lo;
-#ifdef __CUDA_ARCH__
-    const float y = rsqrtf(x);
-#else
-    const float y = 1.f / sqrtf(x);
-#endif
-    const float g = TWA_MUL(x, y);
-    return F2{g, 0.5f * y * (fmaf(-g, g, x) + xl)};
+    RadiusWord w;
+    w.T = rec[F >> 25];
+    w.mh = vfma((float)(F >> 9), 0x1p-23f, 1.f);
+    w.ml = (float)(F & 511u) * 0x1p-32f;
+    w.E = (float)(n + 1 - 33) + w.T.w;
+    return w;
+}
+struct DirectionWord {  // angle = table direction + rest 2 pi / 2^33
+    float rest;
+    float4 D;
+};
+TWA_HD DirectionWord direction_word(uint32_t c, const float4* dir) {
+    // a = 2 c + 1 units of 2 pi / 2^33: the nearest multiple of 2^25 units, |rest| <= 2^24 (exact in a float)
+    const uint32_t j = (c + (1u << 23)) >> 24;       // 0..255, and 0 again past the last (wraps)
+    return {(float)(2 * (int32_t)(c - (j << 24)) + 1), dir[j]};
 }
 
-// cos and sin of 2 pi u, u = (c + 1/2) / 2^32.
-__host__ __device__ __forceinline__ void bm_direction(uint32_t c, const float4* dir, F2& co, F2& si) {
-    // a = 2 c + 1 units of 2 pi / 2^33: the nearest multiple of 2^25 units, |rest| <= 2^24 (exact in a float)
-    const uint32_t j = (c + (1u << 23)) >> 24;               // 0..255, and 0 again past the last (wraps)
-    const float rest = (float)(2 * (int32_t)(c - (j << 24)) + 1);
-    const float4 D = dir[(c + (1u << 23) < c) ? 0 : j];
-    const float kh = 0x1.921fb6p-31f, kl = -0x1.777a5cp-56f; // 2 pi / 2^33
-    const float dh = TWA_MUL(rest, kh), dl = fmaf(rest, kh, -dh) + rest * kl;
-    const float d2 = TWA_MUL(dh, dh);
-    const float d2l = fmaf(dh, dh, -d2) + 2.f * dh * dl;
-    // sin d = dh + sl, cos d = 1 + ch + cl
-    const float sl = fmaf(dh * d2, fmaf(d2, 1.f / 120.f, -1.f / 6.f), dl);
-    const float ch = -0.5f * d2;
-    const float cl = fmaf(d2 * d2, fmaf(d2, -1.f / 720.f, 1.f / 24.f), -0.5f * d2l);
-    auto turn = [&](float ah, float al, float bh, float bl) {  // a cos d + b sin d
-        const float p = TWA_MUL(bh, dh);
-        const float pl = fmaf(bh, dh, -p) + fmaf(bh, sl, bl * dh);
-        const float q = TWA_MUL(ah, ch);
-        const float ql = fmaf(ah, ch, -q) + ah * cl;
-        const F2 s = two_sum(ah, p);
-        const F2 t = two_sum(s.hi, q);
-        return fast_two_sum(t.hi, (s.lo + t.lo) + ((al + pl) + ql));
+// sqrt(-2 ln u) from m = mh + ml, the table's r and -ln r (th + tl), and E.
+template <class V>
+TWA_HD Pair<V> bm_radius(V mh, V ml, V r, V th, V tl, V E) {
+    // m r - 1: both terms exact (|f| < 2^-7, r of 8 bits), then ordered
+    const Pair<V> f = two_sum(vfma(mh, r, vset<V>(-1.f)), vmul(ml, r));
+    // log(1 + f) = f - f^2 / 2 + f^3 (1/3 - f/4 + f^2/5 - f^3/6 + f^4/7)
+    const V f2 = vmul(f.hi, f.hi), f2l = vfma(vadd(f.hi, f.hi), f.lo, vfma(f.hi, f.hi, vneg(f2)));
+    const V p = vfma(f.hi, vfma(f.hi, vfma(f.hi, vfma(f.hi, vset<V>(1.f / 7.f), vset<V>(-1.f / 6.f)), vset<V>(0.2f)),
+                                vset<V>(-0.25f)), vset<V>(1.f / 3.f));
+    const V tail = vfma(vmul(f.hi, f2), p, vfma(vset<V>(-0.5f), f2l, f.lo));
+    const Pair<V> l = fast_two_sum(f.hi, vmul(vset<V>(-0.5f), f2));
+    // ln u = E ln 2 - ln r + log(1 + f); ln 2 as 15 bits (E ln2_hi is exact) and the rest
+    const Pair<V> s0 = fast_two_sum(vmul(E, vset<V>(0x1.62e4p-1f)), th);   // |E ln 2| >= |ln r| or E = 0
+    const Pair<V> s1 = two_sum(s0.hi, l.hi);
+    const V lo = vadd(vadd(vadd(s0.lo, s1.lo), vadd(l.lo, tail)), vfma(E, vset<V>(0x1.7f7d1cp-20f), tl));
+    const Pair<V> L = fast_two_sum(s1.hi, lo);
+    const V x = vmul(vset<V>(-2.f), L.hi), xl = vmul(vset<V>(-2.f), L.lo);
+    const V y = vrsqrt(x);
+    const V g = vmul(x, y);
+    return {g, vmul(vmul(vset<V>(0.5f), y), vadd(vfma(vneg(g), g, x), xl))};
+}
+
+// cos and sin of the angle: directions (ch + cl, sh + sl) of the table turned by rest 2 pi / 2^33.
+template <class V>
+TWA_HD void bm_direction(V rest, V ch, V cl, V sh, V sl, Pair<V>& co, Pair<V>& si) {
+    const V kh = vset<V>(0x1.921fb6p-31f), kl = vset<V>(-0x1.777a5cp-56f);  // 2 pi / 2^33
+    const V dh = vmul(rest, kh), dl = vfma(rest, kl, vfma(rest, kh, vneg(dh)));
+    const V d2 = vmul(dh, dh);
+    const V d2l = vfma(vadd(dh, dh), dl, vfma(dh, dh, vneg(d2)));
+    // sin d = dh + ds, cos d = 1 + qh + ql
+    const V ds = vfma(vmul(dh, d2), vfma(d2, vset<V>(1.f / 120.f), vset<V>(-1.f / 6.f)), dl);
+    const V qh = vmul(vset<V>(-0.5f), d2);
+    const V ql = vfma(vmul(d2, d2), vfma(d2, vset<V>(-1.f / 720.f), vset<V>(1.f / 24.f)), vmul(vset<V>(-0.5f), d2l));
+    auto turn = [&](V ah, V al, V bh, V bl) {  // a cos d + b sin d
+        const V p = vmul(bh, dh);
+        const V pl = vadd(vfma(bh, dh, vneg(p)), vfma(bh, ds, vmul(bl, dh)));
+        const V q = vmul(ah, qh);
+        const V e = vfma(ah, ql, vfma(ah, qh, vneg(q)));
+        const Pair<V> s = two_sum(ah, p);
+        const Pair<V> t = two_sum(s.hi, q);
+        return fast_two_sum(t.hi, vadd(vadd(s.lo, t.lo), vadd(vadd(al, pl), e)));
     };
-    co = turn(D.x, D.y, -D.z, -D.w);
-    si = turn(D.z, D.w, D.x, D.y);
+    co = turn(ch, cl, vneg(sh), vneg(sl));
+    si = turn(sh, sl, ch, cl);
 }
 
 // (a.hi + a.lo) + (b.hi + b.lo), rounded to float once more than exactly
-__host__ __device__ __forceinline__ float add22_round(F2 a, F2 b) {
-    const F2 s = two_sum(a.hi, b.hi);
-    return s.hi + (s.lo + (a.lo + b.lo));
+template <class V>
+TWA_HD V add22_round(Pair<V> a, Pair<V> b) {
+    const Pair<V> s = two_sum(a.hi, b.hi);
+    return vadd(s.hi, vadd(s.lo, vadd(a.lo, b.lo)));
 }
 
 }  // namespace twa
