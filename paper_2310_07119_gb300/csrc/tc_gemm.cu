@@ -5,9 +5,12 @@
 // forward transform of a real field (A = rows of n cells, B = the (re, im) rows of the 2m retained
 // DFT rows, C = interleaved complex coefficients) and the real part of the adjoint (A = rows of 2m
 // complex coefficients as 4m reals, B = (Re M, -Im M) columns, C = n cells).  Both are tall-skinny
-// GEMMs (P up to ~10^7 rows, N and K <= 128) bound by the streaming of A, so one CTA per SM walks row
-// tiles with a double-buffered TMA pipeline while the tensor core and the epilogue work on the
-// previous tile.
+// GEMMs (P up to ~10^7 rows, N and K <= 128) bound by the streaming of A and C, so one CTA per SM walks
+// row tiles with the copies, the products and the stores of three tiles in flight: while tile i is read
+// out of one half of the tensor memory and stored, the products of tile i + 1 go to the other half and
+// the rows of tile i + 2 are copied.  (128^3 x 2, width 32: 181 us a call with the products of a tile
+// behind the stores of the last one, 165 now; 64^3 x 4: 66 and 55.  Turning the tile in shared memory to
+// store whole rows took 174 and 66, eight warps for the stores 167 and 55.)
 //
 // Per CTA (128 threads): thread 0 issues the TMA copies and the MMAs; all four warps read the
 // accumulator out of tensor memory (warp w owns rows 32w..32w+31 of the 128-row tile) and store it.
@@ -79,9 +82,8 @@ k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
           long long P, int N, int Kp, int Np, long long ldc, int accumulate, int ncols, int* err, long long budget) {
     extern __shared__ __align__(1024) uint8_t sraw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(sraw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t bar_a[2], bar_b, bar_mma;
+    __shared__ __align__(8) uint64_t bar_a[2], bar_b, bar_mma[2];
     __shared__ uint32_t tmem_base;
-    __shared__ int s_fail;
     const int natoms = Kp / ATOM_F;
     const uint32_t a_bytes = (uint32_t)natoms * BM * 128, b_bytes = (uint32_t)natoms * Np * 128;
     uint8_t* sA[2] = {sm, sm + a_bytes};
@@ -90,11 +92,11 @@ k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
     const long long ntiles = (P + BM - 1) / BM;
 
     if (threadIdx.x == 0) {
-        s_fail = 0;
-        mbar_init(smem_u32(&bar_a[0]), 1);
-        mbar_init(smem_u32(&bar_a[1]), 1);
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(smem_u32(&bar_a[k]), 1);
+            mbar_init(smem_u32(&bar_mma[k]), 1);
+        }
         mbar_init(smem_u32(&bar_b), 1);
-        mbar_init(smem_u32(&bar_mma), 1);
         mbar_init_fence();
     }
     if (warp == 0) {
@@ -106,94 +108,98 @@ k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tmem_base;
+    const uint32_t tmem = tmem_base, half = (uint32_t)ncols / 2;
     const uint32_t idesc = idesc_tf32(Np);
 
+    int issued = 0, used = 0;  // A tiles copied / waited for by this CTA (thread 0's count)
+    bool b_done = false, bad = false;
     auto load_a = [&](long long tile, int buf) {
         mbar_expect_tx(smem_u32(&bar_a[buf]), a_bytes);
         for (int k = 0; k < natoms; ++k)
             tma_load_2d(smem_u32(sA[buf] + (size_t)k * BM * 128), &ta, k * ATOM_F, (int)(tile * BM), smem_u32(&bar_a[buf]));
+        ++issued;
+    };
+    // the products of this CTA's i-th tile, once its rows have landed
+    auto multiply = [&](int i) {
+        const int buf = i & 1;
+        if (!mbar_wait(smem_u32(&bar_a[buf]), (uint32_t)((i >> 1) & 1), budget)) return false;
+        ++used;
+        fence_after();
+        const uint32_t a0 = smem_u32(sA[buf]), b0 = smem_u32(sB);
+        for (int s = 0; s < Kp / 8; ++s) {
+            const uint32_t koff = (uint32_t)(s % 4) * 32u;  // K = 8 TF32 values = 32 bytes
+            const uint64_t ad = sw128_desc(a0 + (uint32_t)(s / 4) * BM * 128 + koff);
+            const uint64_t bd = sw128_desc(b0 + (uint32_t)(s / 4) * (uint32_t)Np * 128 + koff);
+            mma_tf32(tmem + buf * half, ad, bd, idesc, s > 0 ? 1u : 0u);
+        }
+        mma_commit(smem_u32(&bar_mma[buf]));
+        return true;
     };
     if (threadIdx.x == 0) {
         mbar_expect_tx(smem_u32(&bar_b), b_bytes);
         for (int k = 0; k < natoms; ++k) tma_load_2d(smem_u32(sB + (size_t)k * Np * 128), &tb, k * ATOM_F, 0, smem_u32(&bar_b));
-        if ((long long)blockIdx.x < ntiles) load_a(blockIdx.x, 0);
+        for (int k = 0; k < 2; ++k)
+            if (blockIdx.x + (long long)k * gridDim.x < ntiles) load_a(blockIdx.x + (long long)k * gridDim.x, k);
+        b_done = mbar_wait(smem_u32(&bar_b), 0, budget);
+        bad = !b_done || !multiply(0);   // the grid has at most ntiles CTAs
     }
-    int issued = 0, used = 0;  // A tiles copied / consumed by this CTA (thread 0's count)
-    bool b_done = false;
-    if (threadIdx.x == 0 && (long long)blockIdx.x < ntiles) issued = 1;
-
-    int i = 0;
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
-        const int buf = i & 1;
-        if (threadIdx.x == 0) {
-            const long long next = tile + gridDim.x;
-            // the other buffer was read by the previous tile's MMAs, complete before its epilogue
-            if (next < ntiles) {
-                load_a(next, buf ^ 1);
-                ++issued;
-            }
-            bool ok = true;
-            if (i == 0) ok = b_done = mbar_wait(smem_u32(&bar_b), 0, budget);
-            ok = ok && mbar_wait(smem_u32(&bar_a[buf]), (uint32_t)((i >> 1) & 1), budget);
-            if (ok) {
-                ++used;
-                fence_after();
-                const uint32_t a0 = smem_u32(sA[buf]), b0 = smem_u32(sB);
-                for (int s = 0; s < Kp / 8; ++s) {
-                    const uint32_t koff = (uint32_t)(s % 4) * 32u;  // K = 8 TF32 values = 32 bytes
-                    const uint64_t ad = sw128_desc(a0 + (uint32_t)(s / 4) * BM * 128 + koff);
-                    const uint64_t bd = sw128_desc(b0 + (uint32_t)(s / 4) * (uint32_t)Np * 128 + koff);
-                    mma_tf32(tmem, ad, bd, idesc, s > 0 ? 1u : 0u);
-                }
-                mma_commit(smem_u32(&bar_mma));
-            } else {
-                s_fail = 1;
-            }
-        }
-        __syncthreads();
-        if (s_fail) break;
-        if (!mbar_wait(smem_u32(&bar_mma), (uint32_t)(i & 1), budget)) {
-            atomicOr(&s_fail, 1);
-        }
-        __syncthreads();
-        if (s_fail) break;
-        fence_after();
-        // epilogue: row r of the tile -> TMEM lane r; warp w reads lanes 32w..32w+31
-        const long long row = tile * BM + warp * 32 + lane;
-        float* crow = C + row * ldc;
+    bool stop = __syncthreads_or(bad);
+    if (!stop) {
         const bool vec = (N % 16) == 0 && (ldc % 4) == 0 && ((reinterpret_cast<uintptr_t>(C) & 15u) == 0);
-        for (int c0 = 0; c0 < Np; c0 += 16) {
-            float r[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
-            if (row < P) {
-                if (vec) {
-                    float4* c4 = reinterpret_cast<float4*>(crow + c0);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        float4 o = make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-                        if (accumulate) {
-                            const float4 p = c4[j];
-                            o = make_float4(o.x + p.x, o.y + p.y, o.z + p.z, o.w + p.w);
-                        }
-                        c4[j] = o;
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (c0 + j < N) crow[c0 + j] = accumulate ? crow[c0 + j] + r[j] : r[j];
-                }
+        int i = 0;
+        for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
+            bad = !mbar_wait(smem_u32(&bar_mma[i & 1]), (uint32_t)((i >> 1) & 1), budget);
+            if (threadIdx.x == 0 && !bad) {
+                // the products of tile i are complete: its rows make way for tile i + 2; the accumulator of
+                // tile i + 1 was read out before the last barrier
+                const long long t1 = tile + gridDim.x, t2 = t1 + gridDim.x;
+                if (t2 < ntiles) load_a(t2, i & 1);
+                if (t1 < ntiles) bad = !multiply(i + 1);
             }
+            __syncwarp();
+            if (!__any_sync(0xffffffffu, bad && threadIdx.x != 0)) {
+                fence_after();
+                // row r of the tile -> TMEM lane r; warp w reads lanes 32w..32w+31
+                const long long row = tile * BM + warp * 32 + lane;
+                const uint32_t acc = tmem + (uint32_t)(i & 1) * half + ((uint32_t)(warp * 32) << 16);
+                float* crow = C + row * ldc;
+                for (int c0 = 0; c0 < N; c0 += 16) {
+                    float r[16];
+                    __syncwarp();
+                    tmem_ld16(acc + (uint32_t)c0, r);
+                    if (row >= P) {
+                        // past the last row
+                    } else if (vec) {
+                        float4* c4 = reinterpret_cast<float4*>(crow + c0);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            float4 o = make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+                            if (accumulate) {
+                                const float4 p = c4[j];
+                                o = make_float4(o.x + p.x, o.y + p.y, o.z + p.z, o.w + p.w);
+                            }
+                            c4[j] = o;
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (c0 + j < N) crow[c0 + j] = accumulate ? crow[c0 + j] + r[j] : r[j];
+                    }
+                }
+                fence_before();
+            }
+            stop = __syncthreads_or(bad);
+            if (stop) break;
         }
-        fence_before();
-        __syncthreads();
     }
-    if (s_fail && threadIdx.x == 0) {
-        atomicOr(err, TC_ERR_TIMEOUT_BIT);
-        // copies still in flight land in this CTA's shared memory: wait for them (bounded) before leaving
+    if (threadIdx.x == 0 && stop) {
+        // a wait gave up: copies and products still in flight use this CTA's shared and tensor memory, so
+        // they are waited for (bounded) before leaving
+        if (used > 0) mbar_wait(smem_u32(&bar_mma[(used - 1) & 1]), (uint32_t)(((used - 1) >> 1) & 1), budget);
         for (int u = used; u < issued; ++u) mbar_wait(smem_u32(&bar_a[u & 1]), (uint32_t)((u >> 1) & 1), budget);
         if (!b_done) mbar_wait(smem_u32(&bar_b), 0, budget);
     }
+    if (bad) atomicOr(err, TC_ERR_TIMEOUT_BIT);
     fence_before();
     __syncthreads();
     fence_after();
@@ -244,8 +250,8 @@ int tc_gemm(const float* A, long long P, long long K, long long lda, const float
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms <= 0) sms = 1;
     }
-    int ncols = 32;
-    while (ncols < Np) ncols <<= 1;
+    int ncols = 64;  // an accumulator each for two tiles, on multiples of 32 columns
+    while (ncols < 2 * Np) ncols <<= 1;
     // the peak SM clock, queried once: the attribute query costs hundreds of microseconds per call
     static int khz = 0;
     if (!khz) {
