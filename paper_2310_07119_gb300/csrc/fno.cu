@@ -948,17 +948,38 @@ int twa_fno_create(twa_fno** out, const twa_fno_config* cfg, uint64_t seed) {
     // initial weights: uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) for pointwise maps, scale 1/(W^2) for R,
     // zero biases, from a fixed linear-congruential stream of the seed (host side)
     std::vector<float> h0((size_t)o, 0.f);
-    uint64_t st = seed * 6364136223846793005ULL + 1442695040888963407ULL;
-    auto uni = [&]() {
-        st = st * 6364136223846793005ULL + 1442695040888963407ULL;
-        return ((double)(st >> 11) / 9007199254740992.0) * 2.0 - 1.0;
+    // (eight steps of the stream at a time, each lane jumping eight: one step after the other is a chain
+    // of multiplications, 0.4 s for the 268 M weights of width 32 and 16 modes)
+    constexpr uint64_t A = 6364136223846793005ULL, Cc = 1442695040888963407ULL;
+    uint64_t st = seed * A + Cc;
+    auto fill = [&](long long at, long long n, double div) {
+        constexpr int LN = 8;
+        uint64_t x[LN], a8 = 1, c8 = 0;
+        for (int k = 0; k < LN; ++k) {
+            c8 = c8 * A + Cc;
+            a8 *= A;
+            x[k] = st * a8 + c8;   // the k + 1st next value
+        }
+        float* d = h0.data() + at;
+        auto value = [&](uint64_t v) { return (float)((((double)(v >> 11) / 9007199254740992.0) * 2.0 - 1.0) / div); };
+        long long i = 0;
+        for (; i + LN <= n; i += LN)
+            for (int k = 0; k < LN; ++k) {
+                d[i + k] = value(x[k]);
+                st = x[k];
+                x[k] = x[k] * a8 + c8;
+            }
+        for (int k = 0; i < n; ++i, ++k) {
+            d[i] = value(x[k]);
+            st = x[k];
+        }
     };
-    for (long long i = 0; i < (long long)W * c.c_in; ++i) h0[f->oP + i] = (float)(uni() / std::sqrt((double)c.c_in));
+    fill(f->oP, (long long)W * c.c_in, std::sqrt((double)c.c_in));
     for (int l = 0; l < L; ++l) {
-        for (long long i = 0; i < Mm * W * W * 2; ++i) h0[f->oR[l] + i] = (float)(uni() / ((double)W * W));
-        for (long long i = 0; i < (long long)W * W; ++i) h0[f->oW[l] + i] = (float)(uni() / std::sqrt((double)W));
+        fill(f->oR[l], Mm * W * W * 2, (double)W * W);
+        fill(f->oW[l], (long long)W * W, std::sqrt((double)W));
     }
-    for (long long i = 0; i < (long long)c.c_out * W; ++i) h0[f->oQ + i] = (float)(uni() / std::sqrt((double)W));
+    fill(f->oQ, (long long)c.c_out * W, std::sqrt((double)W));
     cudaMemcpy(f->th, h0.data(), o * sizeof(float), cudaMemcpyHostToDevice);
     k_to_bf16<<<blocks_for(o), kThreads>>>(f->th, f->th16, o);
     cudaMemset(f->am, 0, o * sizeof(float));
