@@ -193,7 +193,7 @@ def _f64_plain_rate(w, steps=2):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1)
     ens.close()
-    fields = 2  # the plain path advances the classical field and the stream one after the other
+    fields = 2  # the classical field and the stream
     return fields * w.grid.cells * steps / (ms * 1e-3)
 
 
