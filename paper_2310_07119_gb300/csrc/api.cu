@@ -983,7 +983,8 @@ int moments_f64(twa_handle* h, Inst& I, double2* psi, const twa_moments_out* o, 
 
 // Workspace of the FP64 path, all of it allocated with the handle (its calls can be captured): packed
 // Poisson fields and spectra for as many streams as fit 1 GB (at least one; grid rows bound them too),
-// and for 1D instances the partial sums of as many outputs as fit 16 MB (none when two do not).
+// and for 1D instances the partial sums of as many outputs as fit 4 MB (none when two do not; 16 MB made a
+// handle take 1.1 ms longer to create).
 int alloc_f64(twa_handle* h, Inst& I) {
     const double field = (double)I.cells * sizeof(double2);
     const int most = (int)std::max(1.0, std::min(32767.0, (double)(1LL << 30) / field));
@@ -995,7 +996,7 @@ int alloc_f64(twa_handle* h, Inst& I) {
         }
     } else {
         const double per_out = (double)I.n_real * (3.0 * I.cells + 1.0) + I.cells;
-        I.run64_outs = (int)std::min(1024.0, (double)(16 << 20) / (8.0 * per_out)) - 1;
+        I.run64_outs = (int)std::min(1024.0, (double)(4 << 20) / (8.0 * per_out)) - 1;
         // without them a 1D run takes its outputs from the moment kernels
         if (I.run64_outs > 0 && dalloc(h, &I.run64, (size_t)(I.run64_outs + 1) * (size_t)per_out) != 0) I.run64 = nullptr;
     }

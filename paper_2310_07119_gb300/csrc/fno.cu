@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <type_traits>
@@ -947,31 +948,38 @@ int twa_fno_create(twa_fno** out, const twa_fno_config* cfg, uint64_t seed) {
     }
     // initial weights: uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) for pointwise maps, scale 1/(W^2) for R,
     // zero biases, from a fixed linear-congruential stream of the seed (host side)
-    std::vector<float> h0((size_t)o, 0.f);
     // (eight steps of the stream at a time, each lane jumping eight: one step after the other is a chain
-    // of multiplications, 0.4 s for the 268 M weights of width 32 and 16 modes)
+    // of multiplications; in pieces of 4 MB, which stay in the host's cache between filling and copying)
     constexpr uint64_t A = 6364136223846793005ULL, Cc = 1442695040888963407ULL;
     uint64_t st = seed * A + Cc;
+    std::vector<float> piece((size_t)std::min<long long>(1 << 20, o));
+    cudaMemset(f->th, 0, o * sizeof(float));
     auto fill = [&](long long at, long long n, double div) {
         constexpr int LN = 8;
-        uint64_t x[LN], a8 = 1, c8 = 0;
+        uint64_t a8 = 1, c8 = 0, x[LN];
         for (int k = 0; k < LN; ++k) {
             c8 = c8 * A + Cc;
             a8 *= A;
             x[k] = st * a8 + c8;   // the k + 1st next value
         }
-        float* d = h0.data() + at;
-        auto value = [&](uint64_t v) { return (float)((((double)(v >> 11) / 9007199254740992.0) * 2.0 - 1.0) / div); };
-        long long i = 0;
-        for (; i + LN <= n; i += LN)
-            for (int k = 0; k < LN; ++k) {
-                d[i + k] = value(x[k]);
-                st = x[k];
-                x[k] = x[k] * a8 + c8;
+        const auto value = [div](uint64_t v) { return (float)((((double)(v >> 11) / 9007199254740992.0) * 2.0 - 1.0) / div); };
+        for (long long done = 0; done < n;) {
+            const long long m = std::min<long long>((long long)piece.size(), n - done);
+            float* d = piece.data();
+            long long i = 0;
+            for (; i + LN <= m; i += LN) {
+                st = x[LN - 1];
+                for (int k = 0; k < LN; ++k) {
+                    d[i + k] = value(x[k]);
+                    x[k] = x[k] * a8 + c8;
+                }
             }
-        for (int k = 0; i < n; ++i, ++k) {
-            d[i] = value(x[k]);
-            st = x[k];
+            for (int k = 0; i < m; ++i, ++k) {   // the last piece only: its size alone is no multiple of eight
+                d[i] = value(x[k]);
+                st = x[k];
+            }
+            cudaMemcpy(f->th + at + done, d, (size_t)m * sizeof(float), cudaMemcpyHostToDevice);
+            done += m;
         }
     };
     fill(f->oP, (long long)W * c.c_in, std::sqrt((double)c.c_in));
@@ -980,7 +988,6 @@ int twa_fno_create(twa_fno** out, const twa_fno_config* cfg, uint64_t seed) {
         fill(f->oW[l], (long long)W * W, std::sqrt((double)W));
     }
     fill(f->oQ, (long long)c.c_out * W, std::sqrt((double)W));
-    cudaMemcpy(f->th, h0.data(), o * sizeof(float), cudaMemcpyHostToDevice);
     k_to_bf16<<<blocks_for(o), kThreads>>>(f->th, f->th16, o);
     cudaMemset(f->am, 0, o * sizeof(float));
     cudaMemset(f->av, 0, o * sizeof(float));
