@@ -113,7 +113,7 @@ typedef struct twa_handle twa_handle;
 /* Create a handle for n_inst instances (grids[i], n_real[i] sampled streams each) sharing *p.
    The handle owns its scratch: the Poisson buffer (8 bytes per cell per pair of slots in
    FP32), the spectral scratch when want_modes is set, twiddle and phase tables, and the
-   graph and autotune state; in FP64 the packed Poisson fields and spectra of as many streams at a
+   graph and autotune state; in FP64 the Poisson half fields and spectra of as many streams at a
    time as fit 1 GB each (at least one) and 4 MB of partial sums for 1D runs.  Must be called with
    the target device current.
    Errors: TWA_EINVAL (sizes), TWA_ENOMEM, TWA_ECUDA. */

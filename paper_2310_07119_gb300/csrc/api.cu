@@ -73,9 +73,9 @@ struct Inst {
     double* prt = nullptr;
     double* dker[3] = {nullptr, nullptr, nullptr};
     // FP64 path
-    double2* work64 = nullptr;  // packed Poisson fields of w_pairs pairs (2D, 3D)
+    double2* work64 = nullptr;  // Poisson half fields of w_slots slots (2D, 3D)
     double2* spec64 = nullptr;  // spectra of spec_fields slots
-    int w_pairs = 0, spec_fields = 0;
+    int w_slots = 0, spec_fields = 0;
     double* run64 = nullptr;    // partial sums of run64_outs + 1 outputs of a whole 1D run
     int run64_outs = 0;
     double* acc64 = nullptr;
@@ -961,7 +961,7 @@ int step_batch_f64(twa_handle* h, Inst& I, double2* psi, int n, cudaStream_t st)
         launch_f64_run1d(psi, I.n_slots, geom64(I), tables64(I), mulc64(h, I), kick, 1, n, nullptr, nullptr, nullptr, st,
                          &h->launches);
     else
-        launch_f64_steps(psi, I.work64, I.w_pairs, I.n_slots, geom64(I), tables64(I), mulc64(h, I), kick, n, st,
+        launch_f64_steps(psi, I.work64, I.w_slots, I.n_slots, geom64(I), tables64(I), mulc64(h, I), kick, n, st,
                          &h->launches);
     return 0;
 }
@@ -981,18 +981,20 @@ int moments_f64(twa_handle* h, Inst& I, double2* psi, const twa_moments_out* o, 
     return 0;
 }
 
-// Workspace of the FP64 path, all of it allocated with the handle (its calls can be captured): packed
-// Poisson fields and spectra for as many streams as fit 1 GB (at least one; grid rows bound them too),
+// Workspace of the FP64 path, all of it allocated with the handle (its calls can be captured): Poisson half
+// fields and spectra for as many streams as fit 1 GB (at least one; grid rows bound them too),
 // and for 1D instances the partial sums of as many outputs as fit 4 MB (none when two do not; 16 MB made a
 // handle take 1.1 ms longer to create).
 int alloc_f64(twa_handle* h, Inst& I) {
-    const double field = (double)I.cells * sizeof(double2);
-    const int most = (int)std::max(1.0, std::min(32767.0, (double)(1LL << 30) / field));
+    const auto most = [](long long cells) {
+        return (int)std::max(1.0, std::min(65535.0, (double)(1LL << 30) / ((double)cells * sizeof(double2))));
+    };
     if (I.mode != MODE_1D) {
-        I.w_pairs = std::min(I.n_pairs, most);
-        while (dalloc(h, &I.work64, (size_t)I.w_pairs * I.cells) != 0) {  // fewer at a time when memory is short
-            if (I.w_pairs == 1) return TWA_ENOMEM;
-            I.w_pairs /= 2;
+        const long long wc = f64_half_cells(geom64(I));
+        I.w_slots = std::min(I.n_slots, most(wc));
+        while (dalloc(h, &I.work64, (size_t)I.w_slots * wc) != 0) {  // fewer at a time when memory is short
+            if (I.w_slots == 1) return TWA_ENOMEM;
+            I.w_slots /= 2;
         }
     } else {
         const double per_out = (double)I.n_real * (3.0 * I.cells + 1.0) + I.cells;
@@ -1003,7 +1005,7 @@ int alloc_f64(twa_handle* h, Inst& I) {
     RC(dalloc(h, &I.acc64, (size_t)3 * I.cells));
     RC(dalloc(h, &I.bad64, 1));
     if (h->p.want_modes) {
-        I.spec_fields = std::min(I.n_real, most);
+        I.spec_fields = std::min(I.n_real, most(I.cells));
         while (dalloc(h, &I.spec64, (size_t)I.spec_fields * I.cells) != 0) {
             if (I.spec_fields == 1) return TWA_ENOMEM;
             I.spec_fields /= 2;

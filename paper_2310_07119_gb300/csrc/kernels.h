@@ -53,8 +53,13 @@ struct Tables64 {
     const double* k2[3];      // k_a^2 per axis
 };
 int f64_prepare();            // kernel attributes of the current device; 0 or -3
-// n_steps KDK steps of a synchronized 2D or 3D batch, w_pairs pairs of streams at a time (W: w_pairs fields)
-int launch_f64_steps(double2* psi, double2* W, int w_pairs, int n_slots, const Geom64& g, const Tables64& t, double mulc,
+// elements of the half field of a real 2D or 3D field: N / 2 + 1 planes of the last axis
+inline long long f64_half_cells(const Geom64& g) {
+    const int n = g.n[g.dim - 1];
+    return g.cells / n * (n / 2 + 1);
+}
+// n_steps KDK steps of a synchronized 2D or 3D batch, w_slots streams at a time (W: w_slots half fields)
+int launch_f64_steps(double2* psi, double2* W, int w_slots, int n_slots, const Geom64& g, const Tables64& t, double mulc,
                      double kick, int n_steps, cudaStream_t st, long long* nl);
 // n_out intervals of out_every steps of a synchronized 1D batch; part (or null): [(n_out + 1) n_real][3][N],
 // part_cl [n_out + 1][N], part_bad [(n_out + 1) n_real], as launch_finish_run1d reads them

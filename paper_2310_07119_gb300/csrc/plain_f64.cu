@@ -6,14 +6,16 @@
 //   * Line transforms are Stockham radix-4 (a radix-2 stage first when log2 N is odd) of butterflies
 //     a +- w b in six fused multiply-adds (a + w b, then 2 a - (a + w b)): 3 instructions per value and
 //     radix-2 level instead of 4.  Four values per thread, stages exchanged through shared memory.
-//   * Two streams share one complex Poisson transform (their densities are its real and imaginary
-//     part; the Poisson operator is real), and the kick, the kinetic phase, the density and 1/k^2 are
-//     part of the transform passes.
+//   * A stream's density and potential are real, so two lines of it along the last axis share one complex
+//     transform and the other axes run over the half field of N / 2 + 1 planes; the kick, the kinetic
+//     phase, the density and 1/k^2 are part of the transform passes.  (Two streams as the real and the
+//     imaginary part of one field take as many operations, but a stream that is not finite, or much larger,
+//     then spoils its partner: here every stream has the same bits whatever the others of its batch hold.)
 //   * All streams of a batch run in each launch.  One launch per stream and operation left most SMs
 //     idle: 100 steps of 32 streams of 256 cells took 25,000 launches and 186 ms.
 //   * A 1D field stays on one SM for a whole run (k64_run1d), a stream per CTA.
 // Measured before and after (one GB300): 100 steps of 32 streams of 256 cells, moments every 10,
-// 182.6 -> 1.04 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.18 ms.  A warp's FP64
+// 182.6 -> 1.04 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.22 ms (4.19 with two streams in one transform).  A warp's FP64
 // instruction occupies its scheduler's unit for about 100 cycles whatever its active lanes (from the times
 // of 8 to 2048 cells), which is what is left in both.
 #include <cuda_runtime.h>
@@ -176,25 +178,21 @@ __device__ __forceinline__ void drift4(double2 (&v)[4], Line64& l, const Axis64&
     fft4(v, l, x, true);
 }
 
-// Pair of slots (2p, 2p + 1), p = blockIdx.y: kick with the pair's potentials (re, im of W; spectral
-// along the axis if vinv), then, if drift, the axis' kinetic factor.
-__global__ void __launch_bounds__(512) k64_kick_drift(Axis64 x, double2* psi, const double2* __restrict__ W, int n_slots,
-                                                       double kick, int vinv, int drift) {
+// Slot blockIdx.y of a pass: kick with the potential V that k64_potential left, then, if drift, the axis'
+// kinetic factor (rows: a row's cells have one index on the last axis, so V is all real or all imaginary parts).
+__global__ void __launch_bounds__(512) k64_kick_drift(Axis64 x, double2* psi, const double2* __restrict__ W,
+                                                       long long wcells, double kick, int drift) {
     Line64 l = line_of(x);
-    double2 w[4], v[4];
-    load4(w, W + (long long)blockIdx.y * x.cells, l);
-    if (vinv) fft4(w, l, x, true);
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        const int slot = 2 * blockIdx.y + h;
-        if (slot >= n_slots) break;
-        double2* f = psi + (long long)slot * x.cells;
-        load4(v, f, l);
+    double2 v[4];
+    double2* f = psi + (long long)blockIdx.y * x.cells;
+    const int upper = l.at >= x.cells / 2;
+    const double* V = reinterpret_cast<const double*>(W + (long long)blockIdx.y * wcells) + upper;
+    const long long at = l.at - upper * (x.cells / 2);
+    load4(v, f, l);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = kick64(v[r], kick * (h ? w[r].y : w[r].x));
-        if (drift) drift4(v, l, x);
-        store4(v, f, l);
-    }
+    for (int r = 0; r < 4; ++r) v[r] = kick64(v[r], kick * __ldg(&V[2 * (at + (long long)r * l.step)]));
+    if (drift) drift4(v, l, x);
+    store4(v, f, l);
 }
 
 __global__ void __launch_bounds__(512) k64_drift(Axis64 x, double2* psi) {
@@ -206,18 +204,18 @@ __global__ void __launch_bounds__(512) k64_drift(Axis64 x, double2* psi) {
     store4(v, f, l);
 }
 
-// Pair: the axis' kinetic factor (if drift), then the packed densities transformed into W.
-__global__ void __launch_bounds__(512) k64_drift_rho(Axis64 x, double2* psi, double2* __restrict__ W, int n_slots,
+// Last axis of slot blockIdx.y, lines l and l + S / 2 at once (x.lines = S / 2): the axis' kinetic factor (if
+// drift), then both lines' densities a and b, transformed as a + i b and taken apart by their symmetry,
+//   2 A_k = w_k + conj w_-k,   2 B_k = -i (w_k - conj w_-k),
+// into the half field W of N / 2 + 1 planes (the factor 2 is undone by the Poisson multiplier).
+__global__ void __launch_bounds__(512) k64_drift_rho(Axis64 x, double2* psi, double2* __restrict__ W, long long wcells,
                                                       int drift) {
     Line64 l = line_of(x);
     double2 v[4], w[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) w[r] = make_double2(0.0, 0.0);
+    const long long other = x.S / 2;
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
-        const int slot = 2 * blockIdx.y + h;
-        if (slot >= n_slots) break;
-        double2* f = psi + (long long)slot * x.cells;
+        double2* f = psi + (long long)blockIdx.y * x.cells + h * other;
         load4(v, f, l);
         if (drift) {
             drift4(v, l, x);
@@ -231,7 +229,45 @@ __global__ void __launch_bounds__(512) k64_drift_rho(Axis64 x, double2* psi, dou
         }
     }
     fft4(w, l, x, false);
-    store4(w, W + (long long)blockIdx.y * x.cells, l);
+    const int q = x.N / 4;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) l.a[pad64(l.j + r * q)] = w[r];
+    __syncthreads();
+    if (!l.act) return;
+    double2* o = W + (long long)blockIdx.y * wcells + l.at;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        if (r == 2 && l.j > 0) break;   // k = j + r N / 4 up to N / 2
+        const double2 c = l.a[pad64((x.N - l.j - r * q) & (x.N - 1))];
+        o[(long long)r * l.step] = make_double2(w[r].x + c.x, w[r].y - c.y);
+        o[(long long)r * l.step + other] = make_double2(w[r].y + c.y, c.x - w[r].x);
+    }
+}
+
+// The way back, in place: lines l and l + S / 2 of the half field to the real potentials V of both lines, cells k
+// and k + N / 2 as the parts of W's element k (so that every line stays within its own elements, all of which its
+// threads have read before the first exchange's barrier).
+__global__ void __launch_bounds__(512) k64_potential(Axis64 x, double2* W, long long wcells) {
+    Line64 l = line_of(x);
+    double2* f = W + (long long)blockIdx.y * wcells + l.at;
+    const long long other = x.S / 2;
+    double2 v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int k = l.j + r * (x.N / 4);
+        const bool conj = k > x.N / 2, real = k == 0 || k == x.N / 2;
+        const long long e = (long long)((conj ? x.N - k : k) - l.j) * x.S;
+        const double2 a = f[e], b = f[e + other];
+        v[r] = real ? make_double2(a.x, b.x)
+                    : (conj ? make_double2(a.x + b.y, b.x - a.y) : make_double2(a.x - b.y, a.y + b.x));
+    }
+    fft4(v, l, x, true);
+    if (!l.act) return;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        f[(long long)r * l.step] = make_double2(v[r].x, v[r + 2].x);
+        f[(long long)r * l.step + other] = make_double2(v[r].y, v[r + 2].y);
+    }
 }
 
 // One field src -> dst (which may be the same): forward (mode 0), inverse (1), or forward, Poisson
@@ -515,53 +551,53 @@ size_t smem64(const Axis64& x) { return 2 * (size_t)x.L * line64(x.N) * sizeof(d
 // 2048 cells in a CTA: two exchange buffers of 36 KB
 int prepare64() {
     for (const void* k : {(const void*)k64_kick_drift, (const void*)k64_drift, (const void*)k64_drift_rho,
-                          (const void*)k64_field})
+                          (const void*)k64_field, (const void*)k64_potential})
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
     if (cudaFuncSetAttribute(k64_run1d<11, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024) != cudaSuccess) return -3;
     return 0;
 }
 
+// cells: of the field, or of the half field of a real one
 void field64(const Geom64& g, const Tables64& t, int a, const double2* src, double2* dst, int n, int mode, double mulc,
-             cudaStream_t st, long long* nl) {
-    const Axis64 x = axis64(g, t, a);
+             long long cells, cudaStream_t st, long long* nl) {
+    Axis64 x = axis64(g, t, a);
+    x.cells = cells;
+    x.lines = cells / x.N;
     const int lx = ilog2(g.n[0]);
     k64_field<<<dim3(tiles64(x), (unsigned)n), threads64(x), smem64(x), st>>>(x, src, dst, mode, lx, lx + ilog2(g.n[1]),
                                                                               t.k2[0], t.k2[1], t.k2[2], mulc);
     ++*nl;
 }
 
-// The rest of the Poisson solve of n packed fields that the last axis' forward transform begins:
-// the potentials in real space (2D), or still spectral along x (3D: the next kick undoes it).
+// The Poisson solve of n half fields between the transforms of the last axis.
 void poisson64(const Geom64& g, const Tables64& t, double2* W, int n, double mulc, cudaStream_t st, long long* nl) {
-    if (g.dim == 2) {
-        field64(g, t, 0, W, W, n, 2, mulc, st, nl);
-        field64(g, t, 1, W, W, n, 1, 0.0, st, nl);
-    } else {
-        field64(g, t, 0, W, W, n, 0, 0.0, st, nl);
-        field64(g, t, 1, W, W, n, 2, mulc, st, nl);
-        field64(g, t, 2, W, W, n, 1, 0.0, st, nl);
-    }
+    const long long wc = f64_half_cells(g);
+    if (g.dim == 3) field64(g, t, 1, W, W, n, 0, 0.0, wc, st, nl);
+    field64(g, t, 0, W, W, n, 2, mulc, wc, st, nl);
+    if (g.dim == 3) field64(g, t, 1, W, W, n, 1, 0.0, wc, st, nl);
 }
 
 }  // namespace
 
 int f64_prepare() { return prepare64(); }
 
-int launch_f64_steps(double2* psi, double2* W, int w_pairs, int n_slots, const Geom64& g, const Tables64& t, double mulc,
+int launch_f64_steps(double2* psi, double2* W, int w_slots, int n_slots, const Geom64& g, const Tables64& t, double mulc,
                      double kick, int n_steps, cudaStream_t st, long long* nl) {
-    const int last = g.dim - 1;
-    for (int s0 = 0; s0 < n_slots; s0 += 2 * w_pairs) {
+    const long long wc = f64_half_cells(g);
+    const Axis64 x0 = axis64(g, t, 0);
+    Axis64 xl = axis64(g, t, g.dim - 1);
+    xl.lines /= 2;   // two at once
+    for (int s0 = 0; s0 < n_slots; s0 += w_slots) {
         double2* f = psi + (size_t)s0 * g.cells;
-        const int ns = n_slots - s0 < 2 * w_pairs ? n_slots - s0 : 2 * w_pairs;
-        const unsigned np = (unsigned)(ns + 1) / 2;
-        const Axis64 x0 = axis64(g, t, 0), xl = axis64(g, t, last);
+        const unsigned ns = (unsigned)(n_slots - s0 < w_slots ? n_slots - s0 : w_slots);
         auto rho = [&](int drift) {
-            k64_drift_rho<<<dim3(tiles64(xl), np), threads64(xl), smem64(xl), st>>>(xl, f, W, ns, drift);
-            ++*nl;
-            poisson64(g, t, W, (int)np, mulc, st, nl);
+            k64_drift_rho<<<dim3(tiles64(xl), ns), threads64(xl), smem64(xl), st>>>(xl, f, W, wc, drift);
+            poisson64(g, t, W, (int)ns, 0.5 * mulc, st, nl);
+            k64_potential<<<dim3(tiles64(xl), ns), threads64(xl), smem64(xl), st>>>(xl, W, wc);
+            *nl += 2;
         };
         auto kicks = [&](double k, int drift) {
-            k64_kick_drift<<<dim3(tiles64(x0), np), threads64(x0), smem64(x0), st>>>(x0, f, W, ns, k, g.dim == 3, drift);
+            k64_kick_drift<<<dim3(tiles64(x0), ns), threads64(x0), smem64(x0), st>>>(x0, f, W, wc, k, drift);
             ++*nl;
         };
         rho(0);
@@ -569,7 +605,7 @@ int launch_f64_steps(double2* psi, double2* W, int w_pairs, int n_slots, const G
             kicks(s == 0 ? 0.5 * kick : kick, 1);
             if (g.dim == 3) {
                 const Axis64 xm = axis64(g, t, 1);
-                k64_drift<<<dim3(tiles64(xm), (unsigned)ns), threads64(xm), smem64(xm), st>>>(xm, f);
+                k64_drift<<<dim3(tiles64(xm), ns), threads64(xm), smem64(xm), st>>>(xm, f);
                 ++*nl;
             }
             rho(1);
@@ -614,7 +650,7 @@ int launch_f64_modes(const double2* psi, double2* spec, int spec_fields, int n_s
     for (int s = 1; s < n_slots; s += spec_fields) {
         const int n = n_slots - s < spec_fields ? n_slots - s : spec_fields;
         for (int a = 0; a < g.dim; ++a)
-            field64(g, t, a, a == 0 ? psi + (size_t)s * g.cells : spec, spec, n, 0, 0.0, st, nl);
+            field64(g, t, a, a == 0 ? psi + (size_t)s * g.cells : spec, spec, n, 0, 0.0, g.cells, st, nl);
         k64_modes_accum<<<ew_blocks(g.cells), 256, 0, st>>>(spec, g.cells, n, anorm2, s == 1, acc2);
         ++*nl;
     }
