@@ -656,7 +656,7 @@ struct twa_fno {
     int npf = 0, npa = 0;
     bool tc_fwd = false, tc_adj = false, tc_on = true;
     int* d_err = nullptr;
-    // activations for the largest batch seen
+    // activations and workspaces for the largest batch seen (held in acts)
     int cap_b = 0;
     std::vector<float*> h, z;   // h[layers] is z[layers - 1]
     std::vector<float2*> s;
@@ -669,7 +669,7 @@ struct twa_fno {
     double* lpart = nullptr;
     const float* x_in = nullptr;
     int last_b = 0;
-    std::vector<void*> allocs;
+    std::vector<void*> allocs, acts;
     std::string err;
 };
 
@@ -688,12 +688,13 @@ int ffail(twa_fno* f, int code, const std::string& m) {
     } while (0)
 
 template <class T>
-int falloc(twa_fno* f, T** p, size_t n) {
+int falloc(twa_fno* f, T** p, size_t n, std::vector<void*>* owner = nullptr) {
     if (cudaMalloc((void**)p, (n ? n : 1) * sizeof(T)) != cudaSuccess) {
         cudaGetLastError();
+        *p = nullptr;
         return ffail(f, TWA_ENOMEM, "twa_fno: cudaMalloc failed");
     }
-    f->allocs.push_back(*p);
+    (owner ? owner : &f->allocs)->push_back(*p);
     return 0;
 }
 
@@ -703,43 +704,48 @@ long long kmodes(const twa_fno* f) {
     return m2 * m2 * m2;
 }
 
+// Free the activations and workspaces of the largest batch seen, and forget the forward that filled them.
+void drop_batch(twa_fno* f) {
+    f->cap_b = f->last_b = 0;
+    f->x_in = nullptr;
+    for (void* p : f->acts) cudaFree(p);
+    f->acts.clear();
+    f->h.clear();
+    f->z.clear();
+    f->s.clear();
+    f->t1 = f->t2 = f->mixed = nullptr;
+    f->dz = f->dz2 = nullptr;
+}
+
+// Room for a batch of B.  When it cannot be had the model holds none at all: a backward is refused, and the
+// next forward starts afresh.
 int ensure_batch(twa_fno* f, int B) {
     if (B <= f->cap_b) return 0;
-    f->cap_b = 0;  // nothing is held if an allocation below fails
-    if (!f->h.empty()) f->h.pop_back();  // z[layers - 1] again
-    for (float* p : f->h) cudaFree(p);
-    for (float* p : f->z) cudaFree(p);
-    for (float2* p : f->s) cudaFree(p);
-    for (void* p : {(void*)f->t1, (void*)f->t2, (void*)f->mixed, (void*)f->dz, (void*)f->dz2})
-        if (p) cudaFree(p);
-    std::vector<void*> keep;
-    for (void* p : f->allocs) {
-        bool act = false;
-        for (float* q : f->h) act |= (p == q);
-        for (float* q : f->z) act |= (p == q);
-        for (float2* q : f->s) act |= (p == (void*)q);
-        for (void* q : {(void*)f->t1, (void*)f->t2, (void*)f->mixed, (void*)f->dz, (void*)f->dz2})
-            act |= (p == q && q);
-        if (!act) keep.push_back(p);
-    }
-    f->allocs = keep;
+    drop_batch(f);
     const int L = f->cfg.layers, W = f->cfg.width, n = f->cfg.grid, m2 = 2 * f->cfg.modes;
-    const long long K = kcells(f), Mm = kmodes(f);
+    const size_t act = (size_t)B * W * kcells(f), modes = (size_t)B * W * kmodes(f);
+    const size_t tsz = (size_t)B * W * n * n * (size_t)(m2 > n ? m2 : n);
     f->h.assign(L, nullptr);
     f->z.assign(L, nullptr);
     f->s.assign(L, nullptr);
-    for (int l = 0; l < L; ++l)
-        if (int rc = falloc(f, &f->h[l], (size_t)B * W * K)) return rc;
+    int rc = 0;
+    auto get = [&](auto** p, size_t count) {
+        if (!rc) rc = falloc(f, p, count, &f->acts);
+    };
+    for (int l = 0; l < L; ++l) get(&f->h[l], act);
     for (int l = 0; l < L; ++l) {
-        if (int rc = falloc(f, &f->z[l], (size_t)B * W * K)) return rc;
-        if (int rc = falloc(f, &f->s[l], (size_t)B * W * Mm)) return rc;
+        get(&f->z[l], act);
+        get(&f->s[l], modes);
     }
-    const size_t tsz = (size_t)B * W * n * n * (size_t)(m2 > n ? m2 : n);
-    if (int rc = falloc(f, &f->t1, tsz)) return rc;
-    if (int rc = falloc(f, &f->t2, tsz)) return rc;
-    if (int rc = falloc(f, &f->mixed, (size_t)B * W * Mm)) return rc;
-    if (int rc = falloc(f, &f->dz, (size_t)B * W * K)) return rc;
-    if (int rc = falloc(f, &f->dz2, (size_t)B * W * K)) return rc;
+    get(&f->t1, tsz);
+    get(&f->t2, tsz);
+    get(&f->mixed, modes);
+    get(&f->dz, act);
+    get(&f->dz2, act);
+    if (rc) {
+        drop_batch(f);
+        return rc;
+    }
     f->h.push_back(f->z[L - 1]);
     f->cap_b = B;
     return 0;
@@ -1002,6 +1008,7 @@ int twa_fno_create(twa_fno** out, const twa_fno_config* cfg, uint64_t seed) {
 
 int twa_fno_destroy(twa_fno* f) {
     if (!f) return TWA_OK;
+    for (void* p : f->acts) cudaFree(p);
     for (void* p : f->allocs) cudaFree(p);
     delete f;
     return TWA_OK;
