@@ -130,6 +130,8 @@ size_t twa_batch_elems(const twa_handle* h);
    precision); slot s >= 1 <- psi_cl + sigma (zR + i zI), with zR, zI standard normals from
    Philox4x32-10 (key = seed, counter = (cell, s, instance, 0)) through Box-Muller in FP64,
    sigma^2 = v / (2 n_tot dV) per real component, v = 1/2 (noise_conv 0) or 1 (noise_conv 1).
+   FP32 fields hold the FP64 values rounded once (most of them formed in float pairs, whose error
+   bound decides the rounding; the others in FP64).
    psi_cl: device complex128, instances concatenated; psi: device batch buffer. */
 int twa_sample(twa_handle* h, const void* psi_cl, uint64_t seed, void* psi, void* stream);
 

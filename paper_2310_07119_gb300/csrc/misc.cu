@@ -39,6 +39,16 @@ __device__ __forceinline__ float2 make_c<float2>(double x, double y) { return ma
 template <>
 __device__ __forceinline__ double2 make_c<double2>(double x, double y) { return make_double2(x, y); }
 
+// z + sigma (zR + i zI), zR, zI from Box-Muller on the Philox words w0, w1, in FP64.
+__device__ __forceinline__ double2 add_noise(double2 z, uint32_t w0, uint32_t w1, double sigma) {
+    const double u0 = ((double)w0 + 0.5) * (1.0 / 4294967296.0);
+    const double u1 = ((double)w1 + 0.5) * (1.0 / 4294967296.0);
+    const double r = sqrt(-2.0 * log(u0));
+    double s, c;
+    sincospi(2.0 * u1, &s, &c);
+    return make_double2(fma(sigma, r * c, z.x), fma(sigma, r * s, z.y));
+}
+
 // Eq. sample: slot 0 <- psi_cl; slot s >= 1 <- psi_cl + sigma (zR + i zI), zR, zI from Box-Muller
 // on the first two Philox words of counter (cell, s, instance, 0), key = seed; arithmetic in FP64.
 template <class T2>
@@ -53,13 +63,7 @@ __global__ void k_sample(const double2* __restrict__ psi_cl, T2* __restrict__ ps
         if (slot > 0) {
             uint32_t c0 = (uint32_t)g, c1 = (uint32_t)slot, c2 = inst, c3 = 0;
             philox4x32_10(c0, c1, c2, c3, k0, k1);
-            const double u0 = ((double)c0 + 0.5) * (1.0 / 4294967296.0);
-            const double u1 = ((double)c1 + 0.5) * (1.0 / 4294967296.0);
-            const double r = sqrt(-2.0 * log(u0));
-            double s, c;
-            sincospi(2.0 * u1, &s, &c);
-            z.x += sigma * (r * c);
-            z.y += sigma * (r * s);
+            z = add_noise(z, c0, c1, sigma);
         }
         psi[idx] = make_c<T2>(z.x, z.y);
     }
@@ -67,15 +71,41 @@ __global__ void k_sample(const double2* __restrict__ psi_cl, T2* __restrict__ ps
 
 __device__ const WignerTables g_wigner = make_wigner_tables();
 
-// The same for float fields: the normals in pairs of floats (wigner.cuh) instead of FP64, each value
-// rounded to float once from about 2^-37.  A thread draws up to `spt` consecutive slots of one cell
+// The value of k_sample, for the few that the float pairs leave open (a call, so that its registers are not the
+// kernel's).
+__device__ __noinline__ float2 sample_f64(double2 z, uint32_t w0, uint32_t w1, double sigma) {
+    z = add_noise(z, w0, w1, sigma);
+    return make_float2((float)z.x, (float)z.y);
+}
+
+// A float that is certainly the rounded sum of a classical value c and a noise n (both pairs), or `open`: where
+// the sum may be on either side of a rounding boundary, or is no finite number.  n is within 1.0e-11 of its exact
+// value, relative (wigner.cuh: radius 2^-40.46, directions 2^-36.64 over all words; sigma and the products far
+// below), which 1.5 2^-37 = 1.09e-11 covers together with the FP64 value's own error and 2^-45 |n| of the sums;
+// ec = 2^-45 |c|, theirs of c.
+struct Rounded {
+    float2 v;
+    bool open_x, open_y;
+};
+__device__ __forceinline__ Rounded round_sum(Pair<float2> c, Pair<float2> n, float ec) {
+    const Pair<float2> s = two_sum(c.hi, n.hi);
+    const float2 t = f2_add(s.lo, f2_add(c.lo, n.lo));
+    const float2 e = make_float2(fmaf(fabsf(n.hi.x), 0x1.8p-37f, ec), fmaf(fabsf(n.hi.y), 0x1.8p-37f, ec));
+    const float2 v = f2_add(s.hi, f2_sub(t, e)), w = f2_add(s.hi, f2_add(t, e));
+    return {v, !(v.x == w.x), !(v.y == w.y)};   // NaN: open
+}
+
+// The same for float fields: the normals in pairs of floats (wigner.cuh) instead of FP64, and the value in FP64
+// only where the pairs do not decide its rounding: every value is that of k_sample, bit for bit.  (The rounded
+// pair sum alone has the same error in the mean, but up to 40 units in the last place where the classical value
+// and the noise cancel.)  A thread draws up to `spt` consecutive slots of one cell
 // (cells = 2^lc), two at a time, so the cell's classical value is split into floats once per spt streams.
 // Bound by the integer and FP32 units (Philox a third of the work); drawing 128^3 x 64 streams took
-// 19.07 ms in FP64, 1.09 ms one value at a time and takes 0.93 to 1.0 ms (its write alone 0.16 ms), with the same
-// error against FP64 (2.5e-8, the rounding).
-__global__ void __launch_bounds__(256)
+// 19.07 ms in FP64 and takes 1.11 ms (noise alone: 1.16), of which the rounding test and its FP64 values are 0.10;
+// the write alone is 0.16.  Open values drawn after the loop: 1.14 and 1.21; three CTAs an SM 1.13, five 1.70.
+__global__ void __launch_bounds__(256, 4)
 k_sample_f32(const double2* __restrict__ psi_cl, float2* __restrict__ psi, int lc, int n_slots, int spt, uint32_t k0,
-             uint32_t k1, uint32_t inst, float sigma, float sigma_lo) {
+             uint32_t k1, uint32_t inst, double sigma) {
     __shared__ WignerTables tab;
     {
         const float4* src = reinterpret_cast<const float4*>(&g_wigner);
@@ -88,11 +118,11 @@ k_sample_f32(const double2* __restrict__ psi_cl, float2* __restrict__ psi, int l
     if (first >= n_slots) return;
     const int last = (int)min((long long)n_slots, first + spt);
     const double2 zc = psi_cl[g];
-    const float hx = (float)zc.x, hy = (float)zc.y;
-    // the remainder of a value that is no finite float is nothing
-    const float rx = isfinite(hx) ? (float)(zc.x - (double)hx) : 0.f, ry = isfinite(hy) ? (float)(zc.y - (double)hy) : 0.f;
+    const float hx = (float)zc.x, hy = (float)zc.y, sh = (float)sigma, sl = (float)(sigma - (double)sh);
+    const float rx = (float)(zc.x - (double)hx), ry = (float)(zc.y - (double)hy);   // NaN for infinities
+    const float ex = fabsf(hx) * 0x1p-45f, ey = fabsf(hy) * 0x1p-45f;
     const Pair<float2> cx{make_float2(hx, hx), make_float2(rx, rx)}, cy{make_float2(hy, hy), make_float2(ry, ry)};
-    const Pair<float2> sg{make_float2(sigma, sigma), make_float2(sigma_lo, sigma_lo)};
+    const Pair<float2> sg{make_float2(sh, sh), make_float2(sl, sl)};
     float2* out = psi + first * cells + g;
     // slots s and s + 1 at once, the lanes of every float2
     for (int s = (int)first; s < last; s += 2, out += 2 * cells) {
@@ -107,11 +137,15 @@ k_sample_f32(const double2* __restrict__ psi_cl, float2* __restrict__ psi, int l
         Pair<float2> co, si;
         bm_direction(make_float2(p.rest, q.rest), make_float2(p.D.x, q.D.x), make_float2(p.D.y, q.D.y),
                      make_float2(p.D.z, q.D.z), make_float2(p.D.w, q.D.w), co, si);
-        const Pair<float2> nx = mul22(r, co), ny = mul22(r, si);
-        const float2 x = add22_round(cx, nx), y = add22_round(cy, ny);
-        // infinities, NaN and overflow: the error terms of the pair sum are no numbers there; slot 0 is psi_cl
-        out[0] = s == 0 ? make_float2(hx, hy) : make_float2(isfinite(x.x) ? x.x : hx + nx.hi.x, isfinite(y.x) ? y.x : hy + ny.hi.x);
-        if (s + 1 < last) out[cells] = make_float2(isfinite(x.y) ? x.y : hx + nx.hi.y, isfinite(y.y) ? y.y : hy + ny.hi.y);
+        const Rounded x = round_sum(cx, mul22(r, co), ex), y = round_sum(cy, mul22(r, si), ey);
+        float2 v0 = make_float2(x.v.x, y.v.x), v1 = make_float2(x.v.y, y.v.y);
+        if (s == 0) v0 = make_float2(hx, hy);   // the classical field
+        else if (x.open_x || y.open_x) v0 = sample_f64(zc, r0, d0, sigma);
+        out[0] = v0;
+        if (s + 1 < last) {
+            if (x.open_y || y.open_y) v1 = sample_f64(zc, r1, d1, sigma);
+            out[cells] = v1;
+        }
     }
 }
 
@@ -553,8 +587,7 @@ int launch_sample_f32(const double2* psi_cl, float2* psi, long long cells, int n
         const long long threads = ((n_slots + spt - 1LL) / spt) * cells, nb = (threads + 255) / 256;
         if (nb < (1LL << 31)) {
             k_sample_f32<<<(unsigned)nb, 256, 0, st>>>(psi_cl, psi, lc, n_slots, spt, (uint32_t)seed,
-                                                       (uint32_t)(seed >> 32), (uint32_t)inst, (float)sigma,
-                                                       (float)(sigma - (double)(float)sigma));
+                                                       (uint32_t)(seed >> 32), (uint32_t)inst, sigma);
             return 0;
         }
     }

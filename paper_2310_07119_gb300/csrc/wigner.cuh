@@ -2,8 +2,8 @@
 //
 // GB300's FP64 rate is 1/64 of its FP32 rate, and the sampled field is stored as floats: a logarithm,
 // a square root and a sine-cosine in FP64 cost 30 times the write of the value.  Here each of them is
-// carried as an unevaluated sum hi + lo of floats, to about 2^-37 relative (far below the 2^-25 of
-// the final rounding to float), from exact integer reductions of the Philox words:
+// carried as an unevaluated sum hi + lo of floats, the radius to 2^-40.4 relative and the directions to 2^-36.6
+// (over all 2^32 words; tests/test_wigner_host.py), from exact integer reductions of the Philox words:
 //   ln u    u = a / 2^33 with a = 2 c + 1, a = m 2^e, 1 <= m < 2: a tabulated 8-bit reciprocal r of
 //           m's interval (top 7 bits), f = m r - 1 exactly as two floats, and the series of
 //           log(1 + f), its first two terms as pairs (the table-driven logarithm of Tang, ACM TOMS
@@ -195,13 +195,6 @@ TWA_HD void bm_direction(V rest, V ch, V cl, V sh, V sl, Pair<V>& co, Pair<V>& s
     };
     co = turn(ch, cl, vneg(sh), vneg(sl));
     si = turn(sh, sl, ch, cl);
-}
-
-// (a.hi + a.lo) + (b.hi + b.lo), rounded to float once more than exactly
-template <class V>
-TWA_HD V add22_round(Pair<V> a, Pair<V> b) {
-    const Pair<V> s = two_sum(a.hi, b.hi);
-    return vadd(s.hi, vadd(s.lo, vadd(a.lo, b.lo)));
 }
 
 }  // namespace twa
