@@ -113,9 +113,10 @@ typedef struct twa_handle twa_handle;
 /* Create a handle for n_inst instances (grids[i], n_real[i] sampled streams each) sharing *p.
    The handle owns its scratch: the Poisson buffer (8 bytes per cell per pair of slots in
    FP32), the spectral scratch when want_modes is set, twiddle and phase tables, and the
-   graph and autotune state; in FP64 the Poisson half fields and spectra of as many streams at a
-   time as fit 1 GB each (at least one) and 4 MB of partial sums for 1D runs.  Must be called with
-   the target device current.
+   graph and autotune state.  In FP64: the Poisson half fields and the spectra of as many streams
+   at a time as fit 1 GB each (one of each instance at least), and for 1D runs 4 to 64 MB of partial
+   sums an instance, up to 1 GB: limits of the whole handle, lower where the GPU would not have
+   room left for a batch.  Must be called with the target device current.
    Errors: TWA_EINVAL (sizes), TWA_ENOMEM, TWA_ECUDA. */
 int twa_create(twa_handle** out, const twa_grid* grids, const twa_params* p,
                int n_inst, const int* n_real);

@@ -76,7 +76,7 @@ struct Inst {
     double2* work64 = nullptr;  // Poisson half fields of w_slots slots (2D, 3D)
     double2* spec64 = nullptr;  // spectra of spec_fields slots
     int w_slots = 0, spec_fields = 0;
-    double* run64 = nullptr;    // partial sums of run64_outs + 1 outputs of a whole 1D run
+    double* run64 = nullptr;    // partial sums of run64_outs + 1 outputs of a whole 1D run (or none)
     int run64_outs = 0;
     double* acc64 = nullptr;
     double* acc64m = nullptr;
@@ -982,38 +982,90 @@ int moments_f64(twa_handle* h, Inst& I, double2* psi, const twa_moments_out* o, 
 }
 
 // Workspace of the FP64 path, all of it allocated with the handle (its calls can be captured): Poisson half
-// fields and spectra for as many streams as fit 1 GB (at least one; grid rows bound them too),
-// and for 1D instances the partial sums of as many outputs as fit 4 MB (none when two do not; 16 MB made a
-// handle take 1.1 ms longer to create).
-int alloc_f64(twa_handle* h, Inst& I) {
-    const auto most = [](long long cells) {
-        return (int)std::max(1.0, std::min(65535.0, (double)(1LL << 30) / ((double)cells * sizeof(double2))));
+// fields and spectra of several streams at a time, and for 1D instances the partial sums of several outputs of a
+// whole run.  One of each field is what a call cannot do without; what goes beyond it is limited for the handle as
+// a whole, shared by its instances in proportion to their streams.
+//   * Fields: 1 GB of each kind fills the GPU's SMs many times over.
+//   * Sums: 4 MB an instance; where these do not hold 16 outputs, those in up to 64 MB.  An instance without them
+//     takes every output from the moment kernels, and one output a launch gains little over that (100 steps, an
+//     output each: 2048 x 60 24.5 ms without, 27.9 one at a time, 11.1 with 16; 256 x 1000 110, 35, 10.2 with 10;
+//     no output 8.4 and 5.6).  An allocation from 2 MB on takes 30 us whatever its size.  Up to 1 GB.
+//   * Never more than a quarter, each, of what the GPU has left beside the least and one batch of the caller's.
+struct F64Share {
+    double poisson, spectra, sums;   // part of what all streams at once would take
+};
+
+long long run64_per_out(const Inst& I) { return (long long)I.n_real * (3 * I.cells + 1) + I.cells; }
+// outputs of a whole 1D run whose sums are wanted at a time, the initial one among them
+long long run64_want(const Inst& I) {
+    const long long bytes = 8 * run64_per_out(I);
+    return std::min(1024LL, std::max((4LL << 20) / bytes, std::min(16LL, (64LL << 20) / bytes)));
+}
+
+int alloc_f64_share(twa_handle* h, const F64Share& sh) {
+    const auto part = [](long long all, double share) {
+        return (int)std::max(1.0, std::min(65535.0, std::floor((double)all * share * (1.0 + 1e-12))));
     };
-    if (I.mode != MODE_1D) {
-        const long long wc = f64_half_cells(geom64(I));
-        I.w_slots = std::min(I.n_slots, most(wc));
-        while (dalloc(h, &I.work64, (size_t)I.w_slots * wc) != 0) {  // fewer at a time when memory is short
-            if (I.w_slots == 1) return TWA_ENOMEM;
-            I.w_slots /= 2;
+    for (auto& I : h->in) {
+        I.run64 = nullptr;
+        I.run64_outs = 0;
+        if (I.mode != MODE_1D) {
+            I.w_slots = part(I.n_slots, std::min(1.0, sh.poisson));
+            RC(dalloc(h, &I.work64, (size_t)I.w_slots * f64_half_cells(geom64(I))));
+        } else {
+            const long long outs = (long long)std::floor((double)run64_want(I) * std::min(1.0, sh.sums) * (1.0 + 1e-12));
+            if (outs >= 2) {
+                RC(dalloc(h, &I.run64, (size_t)outs * (size_t)run64_per_out(I)));
+                I.run64_outs = (int)outs - 1;
+            }
         }
-    } else {
-        const double per_out = (double)I.n_real * (3.0 * I.cells + 1.0) + I.cells;
-        I.run64_outs = (int)std::min(1024.0, (double)(4 << 20) / (8.0 * per_out)) - 1;
-        // without them a 1D run takes its outputs from the moment kernels
-        if (I.run64_outs > 0 && dalloc(h, &I.run64, (size_t)(I.run64_outs + 1) * (size_t)per_out) != 0) I.run64 = nullptr;
-    }
-    RC(dalloc(h, &I.acc64, (size_t)3 * I.cells));
-    RC(dalloc(h, &I.bad64, 1));
-    if (h->p.want_modes) {
-        I.spec_fields = std::min(I.n_real, most(I.cells));
-        while (dalloc(h, &I.spec64, (size_t)I.spec_fields * I.cells) != 0) {
-            if (I.spec_fields == 1) return TWA_ENOMEM;
-            I.spec_fields /= 2;
+        RC(dalloc(h, &I.acc64, (size_t)3 * I.cells));
+        RC(dalloc(h, &I.bad64, 1));
+        if (h->p.want_modes) {
+            I.spec_fields = part(I.n_real, std::min(1.0, sh.spectra));
+            RC(dalloc(h, &I.spec64, (size_t)I.spec_fields * I.cells));
+            RC(dalloc(h, &I.acc64m, (size_t)2 * I.cells));
         }
-        RC(dalloc(h, &I.acc64m, (size_t)2 * I.cells));
     }
-    if (f64_prepare() != 0) return fail(h, TWA_ECUDA, "cudaFuncSetAttribute failed");
     return 0;
+}
+
+int alloc_f64(twa_handle* h) {
+    if (f64_prepare() != 0) return fail(h, TWA_ECUDA, "cudaFuncSetAttribute failed");
+    double least = 0.0, batch = 0.0, poisson = 0.0, spectra = 0.0, sums = 0.0;
+    for (const auto& I : h->in) {
+        const double field = (double)I.cells * sizeof(double2);
+        batch += I.n_slots * field;
+        least += 3.0 * I.cells * sizeof(double);
+        if (I.mode == MODE_1D) {
+            sums += (double)run64_want(I) * (double)run64_per_out(I) * sizeof(double);
+        } else {
+            const double half = (double)f64_half_cells(geom64(I)) * sizeof(double2);
+            least += half;
+            poisson += I.n_slots * half;
+        }
+        if (h->p.want_modes) {
+            least += 2.0 * field;
+            spectra += I.n_real * field;
+        }
+    }
+    size_t free_b = 0, total_b = 0;
+    CU(cudaMemGetInfo(&free_b, &total_b));
+    const size_t mark = h->allocs.size();
+    double room = std::max(0.0, (double)free_b - least - batch) / 4.0;
+    for (;;) {
+        const auto share = [&](double most, double all) { return all > 0.0 ? std::min(most, room) / all : 0.0; };
+        const int rc = alloc_f64_share(
+            h, {share((double)(1LL << 30), poisson), share((double)(1LL << 30), spectra), share((double)(1LL << 30), sums)});
+        if (rc == 0) {
+            h->err.clear();   // of an attempt that took too much
+            return 0;
+        }
+        for (size_t i = mark; i < h->allocs.size(); ++i) cudaFree(h->allocs[i]);
+        h->allocs.resize(mark);
+        if (room == 0.0) return rc;
+        room = room > 64.0 * (1 << 20) ? room / 4.0 : 0.0;
+    }
 }
 
 // Whole 1D FP64 runs: every output's sums come out of the stepping launch (as run1d_all).
@@ -1198,10 +1250,9 @@ int twa_create(twa_handle** out, const twa_grid* grids, const twa_params* p, int
             if ((rc = dalloc(h, &I.vc, (size_t)I.n_pairs * I.cells))) return bail(rc);
             cudaMemset(I.vc, 0, (size_t)I.n_pairs * I.cells * sizeof(float2));
             if (p->want_modes && (rc = dalloc(h, &I.spec, (size_t)I.n_slots * I.cells))) return bail(rc);
-        } else {
-            if ((rc = alloc_f64(h, I))) return bail(rc);
         }
     }
+    if (p->precision == TWA_F64_PLAIN && (rc = alloc_f64(h))) return bail(rc);
     if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_a, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_b, cudaEventDisableTiming) != cudaSuccess) {

@@ -15,7 +15,7 @@ def _cuda():
         pytest.skip("no CUDA device")
 
 
-@pytest.mark.parametrize("n_real,launches", [(20, 6)])     # a stepping and a summing launch for 3 outputs
+@pytest.mark.parametrize("n_real,launches", [(400, 10)])     # a stepping and a summing launch for 2 outputs
 def test_a_run_in_several_launches_equals_its_steps_and_moments(n_real, launches):
     from paper_2310_07119_gb300 import twa_last_launch_count
     n, outs = (2048,), 9
