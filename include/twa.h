@@ -298,8 +298,11 @@ int twa_tc_gemm(const float* A, long long P, long long K, long long lda, const f
                 long long ldc, int accumulate, int* err, void* stream);
 
 /* Block on `stream` and report device-side failures recorded since the last call (TWA_ETIMEOUT: a
-   bounded wait of the persistent launch gave up; TWA_ENONFINITE) or TWA_OK.  Clears the device
-   error word. */
+   bounded wait gave up, of the persistent launch or of a pass whose tiles TMA copies, and the
+   batch's fields are undefined; TWA_ENONFINITE) or TWA_OK.  Clears the device error word.  Tuned
+   handles run such passes where they were fastest, untuned FP32 handles for columns of 1024 and
+   2048 cells and for the 64-cell Poisson columns of 3D grids (a tile's copy takes microseconds, the
+   limit is 2 s; twa_set_wait_limit). */
 int twa_sync_status(twa_handle* h, void* stream);
 
 /* How the instances of a batch run their steps (chosen by twa_autotune, or set here):
