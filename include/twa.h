@@ -202,9 +202,13 @@ int twa_phase_moments(twa_handle* h, int inst, const void* psi, double* var_a, d
 int twa_run(twa_handle* h, const void* psi_cl, uint64_t seed, int n_steps, int out_every,
             void* psi_work, double* series, void* stream);
 
-/* Pass profiler.  While enabled, every FP32 line pass is bracketed by CUDA events on its own
-   stream and graph capture is skipped; twa_profile_read accumulates, per pass kind (op), the
-   number of launches and their total device time in ms since the last enable.  Ops are numbered
+/* Pass profiler.  While enabled, FP32 work runs as line and plane passes one by one, each bracketed
+   by CUDA events on its own stream: no graph capture, no forked or persistent batch, 1D runs
+   interval by interval (a plain call keeps a whole 1D run in one launch), the transforms of the mode
+   moments axis by axis (a plain call fuses the xy transforms of square planes, and the last axis
+   with its sums: the same bits).  twa_profile_read accumulates, per pass kind (op), the number of
+   launches and their total device time in ms since the last enable; the launches of a plain call
+   that are not such passes have no op.  Ops are numbered
    as in the library's pass table (TWA_PROF_NOPS kinds); bytes_per_cell receives the pass's
    algorithmic DRAM traffic in bytes per cell of one launched field (pair or slot). */
 #define TWA_PROF_NOPS 14
