@@ -321,8 +321,8 @@ def _particles_rate(ens, w, n_out=3):
 
 
 def _one_d_rate():
-    """The 1D workload (256 cells, 32 streams + classical, 1000 KDK steps, moments every 10): one
-    on-chip launch per output interval on the FP32 path; the FP64 plain path on the same run."""
+    """The 1D workload (256 cells, 32 streams + classical, 1000 KDK steps, moments every 10): the
+    whole run in one on-chip launch and a finishing one on the FP32 path; the FP64 path on the same run."""
     import torch
     import twa_inputs as ti
     from paper_2310_07119_gb300 import Ensemble, F32, F64_PLAIN, twa_advance
@@ -342,7 +342,7 @@ def _one_d_rate():
         out[name] = w.n_real * w.grid.cells * w.n_steps / (e0.elapsed_time(e1) * 1e-3)
         ens.close()
     return {"value": out["f32"], "f64_plain": out["f64_plain"], "unit": UNIT,
-            "workload": "1D Gaussian bump 256 cells x 32 streams, 1000 KDK steps, moments every 10 (launch- and moment-bound)"}
+            "workload": "1D Gaussian bump 256 cells x 32 streams, 1000 KDK steps, moments every 10 (whole run on chip: instruction latency)"}
 
 
 def _uneven_rate(steps=3):

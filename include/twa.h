@@ -52,6 +52,8 @@ extern "C" {
 
 #define TWA_F32          0   /* batched FP32 path: fused Stockham passes, realization pairs */
 #define TWA_F64_PLAIN    1   /* complex128 fields, every value computed in FP64; all streams in each launch */
+/* Streams that are not finite: in FP64 every stream is computed for itself.  In FP32 slots 2p and
+   2p + 1 share one complex Poisson transform, so a value that is not finite spreads to the partner. */
 
 /* Number of FP64 scalars written per instance per output by twa_moments / twa_run. */
 #define TWA_NSCALARS     8

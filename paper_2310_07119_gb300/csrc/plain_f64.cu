@@ -15,9 +15,10 @@
 //     idle: 100 steps of 32 streams of 256 cells took 25,000 launches and 186 ms.
 //   * A 1D field stays on one SM for a whole run (k64_run1d), a stream per CTA.
 // Measured before and after (one GB300): 100 steps of 32 streams of 256 cells, moments every 10,
-// 182.6 -> 1.04 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.22 ms (4.19 with two streams in one transform).  A warp's FP64
-// instruction occupies its scheduler's unit for about 100 cycles whatever its active lanes (from the times
-// of 8 to 2048 cells), which is what is left in both.
+// 182.6 -> 1.04 ms; 2 steps of one 128^3 stream and its classical field 9.27 -> 4.22 ms.  (Two streams in one
+// transform: 4.18; 32^3 x 16, 50 steps 10.7 ms against 11.1 now, but 512^2 x 8, 20 steps 20.2 against 18.5 and
+// 16^3 x 3, 200 steps 21.7 against 18.6.)  A warp's FP64 instruction occupies its scheduler's unit for about
+// 100 cycles whatever its active lanes (from the times of 8 to 2048 cells), which is what is left in both.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
