@@ -50,7 +50,7 @@ def test_the_batch_has_room_beside_the_workspace():
     n, n_real = (1024, 1024), 88                    # a batch of 1.4 GB; half fields 0.7 GB, spectra 1.4 GB
     torch.cuda.empty_cache()
     batch = (n_real + 1) * n[0] * n[1] * 16
-    fill = torch.empty(torch.cuda.mem_get_info()[0] - batch - _least(n) - GB // 2, dtype=torch.uint8, device="cuda")
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - batch - _least(n) - GB, dtype=torch.uint8, device="cuda")
     ens = _ens([n], [n_real])                       # the handle, then the batch
     ens.psi.fill_(1.0)
     ens.step(1)

@@ -1,7 +1,7 @@
 """The accuracy of the float-pair functions behind the sampling of float fields, held on the host (the same
 arithmetic, one lane): relative errors up to 2^-40.4 of the radius and 2^-36.6 of the directions, which the kernel's
 bound on a value's error is made of (round_sum in misc.cu).  All 2^32 words give 2^-40.463, 2^-36.648 and 2^-36.648
-(nine minutes of one core); here every word where a reduction changes and 2e7 random ones."""
+(a quarter of an hour of one core); here every word where a reduction changes and 2e7 random ones."""
 import math
 import os
 import subprocess
